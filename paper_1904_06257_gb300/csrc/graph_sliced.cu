@@ -1,0 +1,764 @@
+// graph_sliced.cu -- half steps of +-1 graphs at one inverse temperature (anneals, uniform
+// beta), bit-sliced: the 32 replicas of a word are never taken apart.
+//
+// A vertex x of degree d has at most 32 classes of lanes: with a = number of
+// neighbours with J_xy s_y = +1, the threshold T depends on the lane only through
+// idx = a + [sigma = +1] (q = 1, where h(a, +1) = h(a + 1, -1) exactly) or idx = 2 a +
+// [sigma = +1].  One thread owns W group words of a vertex (adjacent in memory).  It
+//   * counts a in bit planes (full adders over the neighbour words, four edges at a
+//     time): 3-4 logic operations per edge and word;
+//   * for each of the top eight threshold planes, selects the class's bit with a tree of
+//     three-input selects over the planes of idx, whose leaves are 0 / ~0 masks taken
+//     from the vertex's class bytes (PRMT with sign replication, shared by the W words);
+//   * compares with the draw's planes least significant first: e = ~(w ^ Q),
+//     lt = e ? lt : Q, eq &= e.
+// Lanes whose top byte equals the threshold's (2^-8), or whose class byte the fp32 bounds
+// do not fix, go one by one to a per-warp queue decided 32 at a time (decide_lane).
+//
+// What bounds it: integer issue.  A LOP3, a PRMT and a wide product each hold the SM
+// quarter's common issue port for two cycles (a product and k logic operations take
+// max(4, 2 + 2k) cycles), so a word of the Erdos-Renyi graph (mean degree 8, n = 10^6,
+// 256 replicas) with its ~300 such operations needs 600 cycles: 120 us a half step, of
+// which 178 us are reached (ALU pipe 56 %, issue 51 %, 1720 warp instructions per
+// 4-word thread, next: gathers).  The general kernel's byte counters, byte lookups and
+// bit transposes take 907 instructions a word and 370 us; with tracking 238 against
+// 412 us.  Four words a thread (16 warps an SM at 128 registers) against two (20 warps):
+// 10.1 against 11.7 ms for 20 tracked steps; against four at 20 warps: 10.6 ms.
+#include <atomic>
+#include <cstdint>
+
+#include "graph_device.cuh"
+#include "shaken_internal.cuh"
+
+namespace shk {
+
+static_assert(kSlicedTile == 128, "four threads per degree 0 .. 31 build the class bytes");
+constexpr int kSlicedQueue = 96;  // queue entries per warp (31 waiting and two per lane)
+constexpr int kSlicedCnt = 10;     // planes of the tracking counters (flushed before 1023)
+constexpr int kSlicedTot = 64;     // groups of a job whose totals a block keeps
+
+struct SlicedShared {
+  // top bytes of T by class, bit-reversed: with one lambda for all vertices by degree, else
+  // by [warp][vertex] of the current tile
+  __align__(16) uint8_t tb[kSlicedTile / 32][32][32];
+  uint32_t amb[32];  // classes of uncertain top byte by degree (one lambda)
+  uint2 key[10];     // Philox round keys
+  uint4 col[kSlicedTile];  // the first four columns of each thread's vertex in the next tile
+  GraphJob J;
+  const uint32_t* src;
+  uint32_t* dst;
+  uint32_t t, typ, skip, fuse, qint, collapse, by_degree;
+  float kb;
+  double beta;
+  unsigned long long dsum;  // degrees of the block's vertices of this job (tracking)
+  uint2 q[kSlicedTile / 32][kSlicedQueue];
+};
+
+template <int W>
+struct SlicedTrack {
+  uint32_t cnt[kSlicedCnt][kSlicedTile][W];       // bit planes of each thread's agreeing-edge counts
+  unsigned int tot[kSlicedTot][32];         // block totals [group of the job][replica lane]
+};
+
+template <int W>
+struct alignas(W == 3 ? 4 : 4 * W) Words {
+  uint32_t v[W];
+};
+
+// The W words from p on: one vector load where rows are a multiple of W words, else words
+// p[min(j, last)] (a row's last thread may have fewer words: the last one again).
+template <int W, bool VEC>
+__device__ __forceinline__ Words<W> ld_words(const uint32_t* p, uint32_t last) {
+  Words<W> r;
+  if constexpr (VEC && W == 4) {
+    const uint4 u = __ldg(reinterpret_cast<const uint4*>(p));
+    r.v[0] = u.x; r.v[1] = u.y; r.v[2] = u.z; r.v[3] = u.w;
+  } else if constexpr (VEC && W == 2) {
+    const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
+    r.v[0] = u.x; r.v[1] = u.y;
+  } else if constexpr (W == 1) {
+    r.v[0] = __ldg(p);
+  } else {
+#pragma unroll
+    for (uint32_t j = 0; j < W; ++j) r.v[j] = __ldg(p + min(j, last));
+  }
+  return r;
+}
+
+template <int W, bool VEC>
+__device__ __forceinline__ void st_words(uint32_t* p, uint32_t last, const uint32_t (&v)[W]) {
+  if constexpr (VEC && W == 4) {
+    *reinterpret_cast<uint4*>(p) = make_uint4(v[0], v[1], v[2], v[3]);
+  } else if constexpr (VEC && W == 2) {
+    *reinterpret_cast<uint2*>(p) = make_uint2(v[0], v[1]);
+  } else {
+#pragma unroll
+    for (uint32_t j = 0; j < W; ++j)
+      if (j <= last) p[j] = v[j];
+  }
+}
+
+__device__ __forceinline__ uint32_t maj3(uint32_t a, uint32_t b, uint32_t c) {
+  return (a & b) | (a & c) | (b & c);
+}
+
+// 0 or ~0: the sign bit of byte B of t, replicated over the word.
+template <int B>
+__device__ __forceinline__ uint32_t byte_sign(uint32_t t) {
+  uint32_t r;
+  asm("prmt.b32 %0, %1, 0, %2;" : "=r"(r) : "r"(t), "n"(0x8888 + 0x1111 * B));
+  return r;
+}
+
+// Selects leaf idx of 2^NB leaves given by the sign bits of the bytes of tb[0 .. 2^NB / 4),
+// for each of W words with idx planes I[b][.].
+template <int NB, int W>
+__device__ __forceinline__ void mux_tree(const uint32_t* tb, const uint32_t (*I)[W],
+                                         uint32_t (&q)[W]) {
+  if constexpr (NB == 2) {
+    const uint32_t m0 = byte_sign<0>(tb[0]), m1 = byte_sign<1>(tb[0]), m2 = byte_sign<2>(tb[0]),
+                   m3 = byte_sign<3>(tb[0]);
+#pragma unroll
+    for (int j = 0; j < W; ++j) {
+      const uint32_t lo = (I[0][j] & m1) | (~I[0][j] & m0);
+      const uint32_t hi = (I[0][j] & m3) | (~I[0][j] & m2);
+      q[j] = (I[1][j] & hi) | (~I[1][j] & lo);
+    }
+  } else {
+    uint32_t lo[W], hi[W];
+    mux_tree<NB - 1, W>(tb, I, lo);
+    mux_tree<NB - 1, W>(tb + (1 << NB) / 8, I, hi);
+#pragma unroll
+    for (int j = 0; j < W; ++j) q[j] = (I[NB - 1][j] & hi[j]) | (~I[NB - 1][j] & lo[j]);
+  }
+}
+
+// What a thread knows about its vertex and words.
+template <int W>
+struct SlicedWord {
+  uint32_t x, go, d, slot;  // vertex, first group of the thread within the job, degree, slot
+  uint32_t last;            // words of the thread beyond the first
+  int p0;
+  bool valid, collapse;
+  uint32_t F;        // frozen mask
+  uint32_t vamb;     // classes of uncertain top byte
+  uint32_t h01[W], l01[W];  // Philox: halves of M0 * u0 of the thread's groups
+  uint32_t c3base;   // update type
+  uint32_t u1;
+};
+
+// The Philox call of planes 4 call .. 4 call + 3 for the thread's W groups (counter words
+// (x, g, t, typ + 2 call)): x, t and the call are common to the words, so round 0 and
+// half of rounds 1 and 2 are computed once (ph_call_shared shares over x instead).
+template <int W>
+__device__ __forceinline__ void sliced_call(const uint2* key, const SlicedWord<W>& w,
+                                            uint32_t c3, uint32_t (&o)[4][W]) {
+  const unsigned long long p0 = (unsigned long long)kPhM0 * w.x;
+  const unsigned long long p1 =
+      (unsigned long long)kPhM1 * ((uint32_t)(p0 >> 32) ^ c3 ^ key[0].y);
+  const uint32_t a0 = (uint32_t)(p1 >> 32) ^ w.u1 ^ key[1].x;
+  const uint32_t a1 = (uint32_t)p1;
+  const unsigned long long q0 = (unsigned long long)kPhM0 * a0;
+#pragma unroll
+  for (int j = 0; j < W; ++j) {
+    const uint32_t c2 = w.h01[j] ^ (uint32_t)p0 ^ key[1].y;
+    const unsigned long long q1 = (unsigned long long)kPhM1 * c2;
+    o[0][j] = (uint32_t)(q1 >> 32) ^ a1 ^ key[2].x;
+    o[1][j] = (uint32_t)q1;
+    o[2][j] = (uint32_t)(q0 >> 32) ^ w.l01[j] ^ key[2].y;
+    o[3][j] = (uint32_t)q0;
+  }
+#pragma unroll
+  for (int r = 3; r < 10; ++r) {
+    const uint2 k = key[r];
+#pragma unroll
+    for (int j = 0; j < W; ++j) {
+      const unsigned long long s0 = (unsigned long long)kPhM0 * o[0][j];
+      const unsigned long long s1 = (unsigned long long)kPhM1 * o[2][j];
+      o[0][j] = (uint32_t)(s1 >> 32) ^ o[1][j] ^ k.x;
+      o[2][j] = (uint32_t)(s0 >> 32) ^ o[3][j] ^ k.y;
+      o[1][j] = (uint32_t)s1;
+      o[3][j] = (uint32_t)s0;
+    }
+  }
+}
+
+// Up to 32 entries of the warp's queue: lane i decides entry i (i < cnt) and sets its bit in
+// the stored word if it is +1.  Entry: (slot, k | idx << 5 | go << 10 | byte << 18 | amb << 26).
+__device__ __noinline__ void sliced_round(const SlicedShared& sh, const uint2* q, int cnt,
+                                             int lane) {
+  __syncwarp();
+  if (lane < cnt) {
+    const uint2 e = q[lane];
+    const GraphJob& J = sh.J;
+    const uint4 vi = __ldg((sh.typ == 0u ? J.in_visit : J.out_visit) + e.x);
+    const int k = (int)(e.y & 31u);
+    const uint32_t idx = (e.y >> 5) & 31u, g = J.g0 + ((e.y >> 10) & 255u);
+    const bool collapse = sh.collapse != 0u;
+    const int a = (int)(collapse ? idx : idx >> 1), sig = collapse ? 0 : (int)(idx & 1u);
+    const int d = (int)vi.z;
+    const float lam = __uint_as_float(vi.w), qf = (float)J.q;
+    const float lmd = __fadd_rn(lam, -(float)d);
+    const float bp = __fadd_rn(lmd, qf), bm = __fadd_rn(lmd, -qf);
+    const float B = (float)d + fabsf(qf) + fabsf(lam) + 1.0f;
+    uint32_t u8 = (e.y >> 18) & 0xFFu;
+    if ((e.y >> 26) & 1u) {  // class of uncertain top byte: the draw's own
+      const PhKey K = ph_key(J.key0, J.key1);
+      const uint4 c0 = ph_call(K, vi.x, g, sh.t, sh.typ), c1 = ph_call(K, vi.x, g, sh.t, sh.typ + 2u);
+      u8 = lane_byte(c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w, k);
+    }
+    if (decide_lane(J.key0, J.key1, vi.x, g, sh.t, sh.typ, k, u8, a, d, sig, bp, bm, J.q, lam,
+                    sh.kb, fabsf(sh.kb) * B, sh.beta, false))
+      atomicOr(sh.dst + (size_t)vi.x * J.G + g, 1u << k);
+  }
+  __syncwarp();
+}
+
+constexpr int kIdx = 5;  // planes of a class index (at most 32 classes)
+
+// Planes 4 call + 3 .. 4 call (least significant first) of the draws o against the
+// thresholds of vertices with at most 2^NB classes.  The call's class bits are the upper
+// (call 1: planes 7..4) or lower four of the bit-reversed bytes.
+template <int NB, int W>
+__device__ __forceinline__ void sliced_planes(const uint8_t* tbv, int call,
+                                              const uint32_t (&I)[kIdx][W], uint32_t (&o)[4][W],
+                                              uint32_t (&lt)[W], uint32_t (&eq)[W]) {
+  constexpr int NW = (1 << NB) / 4;
+  uint32_t tb[NW];
+#pragma unroll
+  for (int k = 0; k < NW; ++k)
+    tb[k] = reinterpret_cast<const uint32_t*>(tbv)[k] << (call != 0 ? 0 : 4);
+  auto plane = [&]() {
+    uint32_t Q[W];
+    mux_tree<NB, W>(tb, I, Q);
+#pragma unroll
+    for (int k = 0; k < NW; ++k) tb[k] <<= 1;
+#pragma unroll
+    for (int j = 0; j < W; ++j) {
+      lt[j] = maj3(~o[3][j], Q[j], lt[j]);
+      eq[j] &= ~(o[3][j] ^ Q[j]);
+      o[3][j] = o[2][j];
+      o[2][j] = o[1][j];
+      o[1][j] = o[0][j];
+    }
+  };
+#pragma unroll 1
+  for (int i = 0; i < 4; ++i) plane();  // a loop, for the instruction cache
+}
+
+// Decisions of the warp's vertices (one tile row); ncls: the most classes among them.
+// Only the plane comparison is compiled once per class width, the rest of the body is
+// common: four whole bodies (119 KB) missed the instruction cache for a third of the stalls.
+template <int W, bool VEC, bool TRACK>
+__device__ __forceinline__ void sliced_decide(SlicedShared& sh, SlicedTrack<W>* tr,
+                                              const SlicedWord<W>& w, const uint8_t* tbv,
+                                              uint32_t ncls, bool have, const uint4* next,
+                                              uint2* q, int& qn, int lane) {
+  const GraphJob& J = sh.J;
+  const uint32_t G = J.G;
+  const uint32_t* src = sh.src + J.g0 + w.go;
+  const uint32_t* col = w.c3base == 0u ? J.in_col : J.out_col;
+  uint32_t I[kIdx][W], S[W];
+#pragma unroll
+  for (int j = 0; j < W; ++j) {
+    S[j] = 0u;
+#pragma unroll
+    for (int b = 0; b < kIdx; ++b) I[b][j] = 0u;
+  }
+  if (w.valid) {
+    const Words<W> own = ld_words<W, VEC>(src + (size_t)w.x * G, w.last);
+#pragma unroll
+    for (int j = 0; j < W; ++j) S[j] = own.v[j];
+    uint32_t cv[4];  // four edges at a time; beyond the degree the last edge again, masked out
+    if (have) {      // copied during the previous tile
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      const uint4 c = sh.col[threadIdx.x];
+      cv[0] = c.x; cv[1] = c.y; cv[2] = c.z; cv[3] = c.w;
+    } else if (w.d != 0u) {
+#pragma unroll
+      for (uint32_t i = 0; i < 4; ++i) cv[i] = __ldg(col + w.p0 + min(i, w.d - 1u));
+    }
+#pragma unroll 1
+    for (uint32_t e = 0; e < w.d; e += 4) {
+      uint32_t x[4][W];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const Words<W> nb = ld_words<W, VEC>(src + (size_t)(cv[i] & 0x7fffffffu) * G, w.last);
+        const uint32_t s = (uint32_t)((int32_t)cv[i] >> 31);  // J < 0
+        const uint32_t m = e + i < w.d ? 0xffffffffu : 0u;
+#pragma unroll
+        for (int j = 0; j < W; ++j) x[i][j] = (nb.v[j] ^ s) & m;
+      }
+      if (e + 4u < w.d) {
+#pragma unroll
+        for (uint32_t i = 0; i < 4; ++i) cv[i] = __ldg(col + w.p0 + min(e + 4u + i, w.d - 1u));
+      }
+      uint32_t c[W];
+#pragma unroll
+      for (int j = 0; j < W; ++j) {
+        const uint32_t s0 = I[0][j] ^ x[0][j] ^ x[1][j], ca = maj3(I[0][j], x[0][j], x[1][j]);
+        const uint32_t cb = maj3(s0, x[2][j], x[3][j]);
+        I[0][j] = s0 ^ x[2][j] ^ x[3][j];
+        const uint32_t cc = maj3(I[1][j], ca, cb);
+        I[1][j] ^= ca ^ cb;
+        c[j] = I[2][j] & cc;
+        I[2][j] ^= cc;
+      }
+      if (ncls > 8u) {  // counts beyond three planes
+#pragma unroll
+        for (int j = 0; j < W; ++j) {
+          I[4][j] ^= I[3][j] & c[j];
+          I[3][j] ^= c[j];
+        }
+      }
+    }
+  }
+  if (next != nullptr && next->z != 0u) {  // the next tile's columns, on their way during the rest
+    const uint32_t at = (uint32_t)__cvta_generic_to_shared(&sh.col[threadIdx.x]);
+#pragma unroll
+    for (uint32_t i = 0; i < 4; ++i)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(at + 4u * i),
+                   "l"(col + next->y + min(i, next->z - 1u))
+                   : "memory");
+  }
+  if (TRACK && sh.fuse) {
+    // agreeing edges (J_xy s_x s_y = +1) per lane: a where sigma = +1, d - a otherwise,
+    // added to the thread's counter planes
+    const uint32_t dd = w.valid ? w.d : 0u;
+    uint32_t br[W], carry[W];
+#pragma unroll
+    for (int j = 0; j < W; ++j) br[j] = carry[j] = 0u;
+#pragma unroll
+    for (int b = 0; b < kIdx; ++b) {
+      const uint32_t D = 0u - ((dd >> b) & 1u);
+      Words<W>& cw = *reinterpret_cast<Words<W>*>(tr->cnt[b][threadIdx.x]);
+      Words<W> c = cw;
+#pragma unroll
+      for (int j = 0; j < W; ++j) {
+        const uint32_t A = I[b][j], df = D ^ A ^ br[j], old = c.v[j];
+        br[j] = (~D & A) | (~D & br[j]) | (A & br[j]);
+        const uint32_t ag = (S[j] & A) | (~S[j] & df);
+        c.v[j] = old ^ ag ^ carry[j];
+        carry[j] = maj3(old, ag, carry[j]);
+      }
+      cw = c;
+    }
+#pragma unroll 1
+    for (int b = kIdx; b < kSlicedCnt; ++b) {
+      Words<W>& cw = *reinterpret_cast<Words<W>*>(tr->cnt[b][threadIdx.x]);
+      Words<W> c = cw;
+      uint32_t any = 0u;
+#pragma unroll
+      for (int j = 0; j < W; ++j) {
+        const uint32_t old = c.v[j];
+        c.v[j] = old ^ carry[j];
+        carry[j] &= old;
+        any |= carry[j];
+      }
+      cw = c;
+      if (any == 0u) break;
+    }
+  }
+  if (w.collapse) {  // idx = a + sigma
+#pragma unroll
+    for (int j = 0; j < W; ++j) {
+      uint32_t c = S[j];
+#pragma unroll
+      for (int b = 0; b < kIdx; ++b) {
+        const uint32_t t = I[b][j] & c;
+        I[b][j] ^= c;
+        c = t;
+      }
+    }
+  } else {  // idx = 2 a + sigma
+#pragma unroll
+    for (int j = 0; j < W; ++j) {
+#pragma unroll
+      for (int b = kIdx - 1; b > 0; --b) I[b][j] = I[b - 1][j];
+      I[0][j] = S[j];
+    }
+  }
+  uint32_t lt[W], eq[W];
+#pragma unroll
+  for (int j = 0; j < W; ++j) {
+    lt[j] = 0u;
+    eq[j] = ~w.F;
+  }
+#pragma unroll 1
+  for (int call = 1; call >= 0; --call) {
+    uint32_t o[4][W];
+    sliced_call<W>(sh.key, w, w.c3base + 2u * (uint32_t)call, o);
+    if (ncls <= 4u)
+      sliced_planes<2, W>(tbv, call, I, o, lt, eq);
+    else if (ncls <= 8u)
+      sliced_planes<3, W>(tbv, call, I, o, lt, eq);
+    else if (ncls <= 16u)
+      sliced_planes<4, W>(tbv, call, I, o, lt, eq);
+    else
+      sliced_planes<5, W>(tbv, call, I, o, lt, eq);
+  }
+  uint32_t cu = 0u;  // lanes left to the queue
+#pragma unroll
+  for (int j = 0; j < W; ++j) {
+    uint32_t amb = 0u;
+#pragma unroll 1
+    for (uint32_t m = w.vamb; m != 0u; m &= m - 1u) {  // rare: lanes of uncertain classes
+      const uint32_t c = (uint32_t)__ffs(m) - 1u;
+      uint32_t is = 0xffffffffu;
+#pragma unroll
+      for (int b = 0; b < kIdx; ++b) is &= ~(I[b][j] ^ (0u - ((c >> b) & 1u)));
+      amb |= is;
+    }
+    eq[j] = w.valid && (VEC || (uint32_t)j <= w.last) ? (eq[j] | amb) & ~w.F : 0u;  // undecided
+    lt[j] = (lt[j] & ~eq[j]) | w.F;
+    cu += (uint32_t)__popc(eq[j]);
+  }
+  if (w.valid) st_words<W, VEC>(sh.dst + J.g0 + w.go + (size_t)w.x * G, w.last, lt);
+  if (!__any_sync(0xffffffffu, cu != 0u)) return;
+  // queue entries of the undecided lanes
+  const uint32_t below = (1u << lane) - 1u;
+  auto entry = [&](int j, int k) {
+    uint32_t idx = 0u;
+#pragma unroll
+    for (int b = 0; b < kIdx; ++b) idx |= ((I[b][j] >> k) & 1u) << b;
+    return make_uint2(w.slot, (uint32_t)k | (idx << 5) | ((w.go + (uint32_t)j) << 10) |
+                                  ((__brev((uint32_t)tbv[idx]) >> 24) << 18) |
+                                  (((w.vamb >> idx) & 1u) << 26));
+  };
+  // places by a prefix sum over the lanes' counts: all of them when they fit, else at most
+  // two of each lane at a time; a round whenever 32 wait
+#pragma unroll 1
+  do {
+    uint32_t c = min(cu, 7u), pos, total;
+    auto places = [&]() {
+      pos = (uint32_t)qn;
+      total = 0u;
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        const uint32_t m = __ballot_sync(0xffffffffu, (c >> b) & 1u);
+        pos += (uint32_t)__popc(m & below) << b;
+        total += (uint32_t)__popc(m) << b;
+      }
+    };
+    places();
+    if (qn + (int)total > kSlicedQueue) {  // uniform
+      c = min(cu, 2u);
+      places();
+    }
+    cu -= c;
+#pragma unroll
+    for (int j = 0; j < W; ++j)
+      while (c != 0u && eq[j] != 0u) {
+        q[pos++] = entry(j, __ffs(eq[j]) - 1);
+        eq[j] &= eq[j] - 1u;
+        --c;
+      }
+    qn += (int)total;
+    while (qn >= 32) {
+      qn -= 32;
+      sliced_round(sh, q + qn, 32, lane);
+    }
+  } while (__any_sync(0xffffffffu, cu != 0u));
+}
+
+// Lane k's column of the warp's 32 words (bit i = bit k of lane i's word).
+__device__ __forceinline__ uint32_t warp_column(uint32_t x, int lane) {
+  const uint32_t Hm[5] = {0xFFFF0000u, 0xFF00FF00u, 0xF0F0F0F0u, 0xCCCCCCCCu, 0xAAAAAAAAu};
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    const int j = 16 >> i;
+    const uint32_t p = __shfl_xor_sync(0xffffffffu, x, j);
+    const bool hi = (lane & j) != 0;
+    const uint32_t t = hi ? (p >> j) : (p << j);
+    const uint32_t M = hi ? ~Hm[i] : Hm[i];
+    x = (x & ~M) | (t & M);
+  }
+  return x;
+}
+
+// The warp's counter planes into the block's totals (or, for jobs of more groups than the
+// block keeps, into the sums), and cleared.
+template <int W>
+__device__ __noinline__ void sliced_flush(SlicedShared& sh, SlicedTrack<W>* tr, int lane) {
+  const GraphJob& J = sh.J;
+  const uint32_t sw = J.sGp < 32u ? J.sGp : 32u;
+  const uint32_t base = ((uint32_t)threadIdx.x & ~31u) & (J.sGp - 1u);
+#pragma unroll 1
+  for (int j = 0; j < W; ++j) {
+    uint32_t col[kSlicedCnt];
+#pragma unroll
+    for (int b = 0; b < kSlicedCnt; ++b) {
+      col[b] = warp_column(tr->cnt[b][threadIdx.x][j], lane);
+      tr->cnt[b][threadIdx.x][j] = 0u;
+    }
+    uint32_t mask = 0u;
+#pragma unroll 1
+    for (uint32_t i = 0; i < 32u; i += sw) mask |= 1u << i;
+#pragma unroll 1
+    for (uint32_t s = 0; s < sw; ++s, mask <<= 1) {
+      uint32_t c = 0u;
+#pragma unroll
+      for (int b = 0; b < kSlicedCnt; ++b) c += (uint32_t)__popc(col[b] & mask) << b;
+      const uint32_t go = (base + s) * W + (uint32_t)j;
+      if (go < J.Gj && c != 0u) {
+        if (J.Gj <= (uint32_t)kSlicedTot)
+          atomicAdd(&tr->tot[go][lane], c);
+        else
+          atomicAdd(J.sums + (size_t)(32u * (J.g0 + go) + (uint32_t)lane) * kNumSums + kSumE,
+                    2.0 * (double)c);
+      }
+    }
+  }
+}
+
+// Class i of a vertex of degree d and field lam: its top byte into tbv[i] (bit-reversed);
+// 1 if the bounds do not fix it.
+__device__ __forceinline__ uint32_t sliced_class(const SlicedShared& sh, uint32_t i, uint32_t d,
+                                                 float lam, uint8_t* tbv) {
+  const uint32_t a = sh.collapse ? i : i >> 1;
+  const bool up = !sh.collapse && (i & 1u) != 0u;
+  const float qf = (float)sh.J.q, fd = (float)d;
+  const float h0 = __fadd_rn(__fadd_rn(lam, -fd), up ? qf : -qf);  // h = 2a + (lambda - d +- q)
+  const float hf = fmaf(2.0f, (float)a, h0);
+  float lo, hi;
+  t_bounds(hf, sh.kb, fabsf(sh.kb) * (fd + fabsf(qf) + fabsf(lam) + 1.0f), lo, hi);
+  uint32_t bl = top_byte(lo), bh = top_byte(hi);
+  // a field of exactly 0 has T = 2^31; with lambda = 0 and an integer q the fp32 field is
+  // exact
+  if (hf == 0.0f &&
+      (lam == 0.0f ? sh.qint != 0u : field_is_zero(2 * (int)a - (int)d, up, sh.J.q, lam)))
+    bl = bh = 0x80u;
+  tbv[i] = (uint8_t)(__brev(bh) >> 24);
+  return bl != bh ? 1u : 0u;
+}
+
+template <int W, bool VEC, bool TRACK>
+__global__ void __launch_bounds__(kSlicedTile, 4) graph_sliced_kernel(
+    const GraphJob* __restrict__ jobs, const Tile* __restrict__ tiles, int n_tiles,
+    uint32_t half) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  SlicedShared& sh = *reinterpret_cast<SlicedShared*>(smem_raw);
+  SlicedTrack<W>* tr = reinterpret_cast<SlicedTrack<W>*>(smem_raw + (sizeof(SlicedShared) + 15) / 16 * 16);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tb = (int)(((long long)blockIdx.x * n_tiles) / gridDim.x);
+  const int te = (int)(((long long)(blockIdx.x + 1) * n_tiles) / gridDim.x);
+  const GraphJob& J = sh.J;
+  int cur_job = -1, qn = 0;
+  uint32_t bound = 0u;  // no counter of the warp exceeds this (warp-uniform)
+  uint2* q = sh.q[warp];
+  SlicedWord<W> w;
+  const uint4* visit = nullptr;
+  bool have = false;  // this thread's columns were copied during the previous tile
+  if (TRACK) {
+#pragma unroll 1
+    for (int i = tid; i < kSlicedTot * 32; i += kSlicedTile) (&tr->tot[0][0])[i] = 0u;
+#pragma unroll
+    for (int b = 0; b < kSlicedCnt; ++b)
+#pragma unroll
+      for (int j = 0; j < W; ++j) tr->cnt[b][tid][j] = 0u;
+  }
+  // the job's queued lanes and tracking sums, before another job is staged
+  auto leave = [&]() {
+    if (qn > 0) sliced_round(sh, q, qn, lane);
+    qn = 0;
+    if (TRACK && sh.fuse) {
+      sliced_flush<W>(sh, tr, lane);
+      bound = 0u;
+      __syncthreads();
+      const double ds = (double)sh.dsum;
+#pragma unroll 1
+      for (uint32_t o = (uint32_t)tid; o < 32u * J.Gj; o += kSlicedTile) {
+        double v = -ds;
+        if (J.Gj <= (uint32_t)kSlicedTot) {
+          v += 2.0 * (double)(&tr->tot[0][0])[o];
+          (&tr->tot[0][0])[o] = 0u;
+        }
+        if (v != 0.0) atomicAdd(J.sums + (size_t)(32u * J.g0 + o) * kNumSums + kSumE, v);
+      }
+    }
+  };
+  Tile tl = tiles[tb], tn;
+  uint4 vi = make_uint4(0u, 0u, 0u, 0u), vn;  // visit entries of this tile and the next
+  for (int ti = tb; ti < te; ++ti, tl = tn, vi = vn) {
+    if (ti + 1 < te) tn = tiles[ti + 1];
+    if ((int)tl.job != cur_job) {
+      if (cur_job >= 0) leave();
+      __syncthreads();  // shared per-job values are about to change
+      if (tid < (int)(sizeof(GraphJob) / 4))
+        reinterpret_cast<uint32_t*>(&sh.J)[tid] =
+            reinterpret_cast<const uint32_t*>(jobs + tl.job)[tid];
+      __syncthreads();
+      if (tid == 0) {
+        const CtxDev* cd = J.cd;
+        const uint32_t t = cd->step;
+        double b0;
+        if (J.beta_sched != nullptr && cd->anneal_len != 0u) {
+          uint32_t k = t - cd->anneal_t0;
+          if (k >= cd->anneal_len) k = cd->anneal_len - 1u;
+          b0 = J.beta_sched[k];
+        } else {
+          b0 = J.beta_lane[32u * J.g0];
+        }
+        const bool skip = t >= cd->t_end;
+        sh.skip = skip ? 1u : 0u;
+        sh.fuse = (TRACK && !skip && half == 0u && cd->tracking && !cd->record &&
+                   J.sums != nullptr) ? 1u : 0u;
+        sh.src = half == 0u ? J.A : J.B;
+        sh.dst = half == 0u ? J.B : J.A;
+        sh.t = t;
+        sh.typ = half ^ cd->order;
+        sh.beta = b0;
+        sh.kb = (float)(-2.0 * b0 * 1.4426950408889634);
+        sh.collapse = J.q == 1.0 ? 1u : 0u;
+        sh.by_degree = J.lambda == nullptr ? 1u : 0u;
+        sh.qint = J.q == rint(J.q) ? 1u : 0u;
+        sh.dsum = 0ull;
+      }
+      __syncthreads();
+      cur_job = (int)tl.job;
+      have = false;
+      visit = sh.typ == 0u ? J.in_visit : J.out_visit;
+      if (tl.w0 + (uint32_t)tid / J.sGp < J.n) vi = __ldg(visit + tl.w0 + (uint32_t)tid / J.sGp);
+      if (tid < 10) sh.key[tid] = make_uint2(J.key0 + (uint32_t)tid * kPhW0, J.key1 + (uint32_t)tid * kPhW1);
+      if (sh.by_degree && !sh.skip) {  // four lanes of a degree's classes each
+        const uint32_t d = (uint32_t)tid >> 2;
+        const uint32_t ncls = sh.collapse ? d + 2u : 2u * d + 2u;
+        uint32_t mine = 0u;
+        for (uint32_t i = (uint32_t)tid & 3u; i < ncls && i < 32u; i += 4u)
+          mine |= sliced_class(sh, i, d, J.lambda_c, &sh.tb[0][0][0] + 32u * d) << i;
+        mine |= __shfl_xor_sync(0xffffffffu, mine, 1);
+        mine |= __shfl_xor_sync(0xffffffffu, mine, 2);
+        if ((tid & 3) == 0) sh.amb[d] = mine;
+      }
+      __syncthreads();
+      w.collapse = sh.collapse != 0u;
+      w.go = ((uint32_t)tid & (J.sGp - 1u)) * W;
+      w.last = w.go < J.Gj ? min((uint32_t)W - 1u, J.Gj - 1u - w.go) : 0u;
+      w.c3base = sh.typ;
+      const unsigned long long p1 = (unsigned long long)kPhM1 * sh.t;
+      w.u1 = (uint32_t)p1;
+#pragma unroll
+      for (int j = 0; j < W; ++j) {
+        const uint32_t u0 = (uint32_t)(p1 >> 32) ^ (J.g0 + w.go + (uint32_t)j) ^ J.key0;
+        const unsigned long long m = (unsigned long long)kPhM0 * u0;
+        w.h01[j] = (uint32_t)(m >> 32);
+        w.l01[j] = (uint32_t)m;
+      }
+    }
+    if (sh.skip) continue;
+    const uint32_t Gp = J.sGp, sw = Gp < 32u ? Gp : 32u, gs = (uint32_t)lane & (sw - 1u);
+    const uint32_t slot = tl.w0 + (uint32_t)tid / Gp;
+    const bool in = slot < J.n;
+    w.slot = slot;
+    w.valid = in && w.go < J.Gj;
+    w.x = in ? vi.x : 0u;
+    w.p0 = in ? (int)vi.y : 0;
+    w.d = in ? vi.z : 0u;
+    const float lam = in ? __uint_as_float(vi.w) : 0.0f;
+    // the next tile's entry, in flight during this one (another job's: read when staged)
+    bool more = false;
+    if (ti + 1 < te && (int)tn.job == cur_job) {
+      const uint32_t ns = tn.w0 + (uint32_t)tid / Gp;
+      more = ns < J.n && w.go < J.Gj;
+      if (ns < J.n) vn = __ldg(visit + ns);
+    }
+    w.F = (in && J.frozen != nullptr) ? __ldg(J.frozen + w.x) : 0u;
+    const uint32_t ncls = !in ? 0u : w.collapse ? w.d + 2u : 2u * w.d + 2u;
+    const uint8_t* tbv;
+    if (sh.by_degree) {
+      const uint32_t d = min(w.d, 31u);
+      tbv = &sh.tb[0][0][0] + 32u * d;
+      w.vamb = sh.amb[d];
+    } else {  // the vertex's threads take turns
+      uint8_t* own = sh.tb[warp][(uint32_t)lane / sw];
+      uint32_t mine = 0u;
+      for (uint32_t i = gs; i < ncls; i += sw)
+        mine |= sliced_class(sh, i, w.d, lam, own) << i;
+      for (uint32_t s = 1u; s < sw; s <<= 1) mine |= __shfl_xor_sync(0xffffffffu, mine, s);
+      w.vamb = mine;
+      tbv = own;
+    }
+    const uint32_t nm = __reduce_max_sync(0xffffffffu, ncls);
+    __syncwarp();
+    if (TRACK && sh.fuse) {
+      const uint32_t dm = __reduce_max_sync(0xffffffffu, w.d);
+      if (bound + dm > (1u << kSlicedCnt) - 1u) {
+        sliced_flush<W>(sh, tr, lane);
+        bound = 0u;
+      }
+      bound += dm;
+      const uint32_t ds = __reduce_add_sync(0xffffffffu, w.valid && w.go == 0u ? w.d : 0u);
+      if (lane == 0 && ds != 0u) atomicAdd(&sh.dsum, (unsigned long long)ds);
+    }
+    sliced_decide<W, VEC, TRACK>(sh, tr, w, tbv, nm, have, more ? &vn : nullptr, q, qn, lane);
+    have = more && vn.z != 0u;
+    __syncwarp();  // the class bytes are read before the next vertices' are written
+  }
+  if (cur_job >= 0 && !sh.skip) leave();
+}
+
+// Dynamic shared memory and resident blocks of a variant on the current device.
+template <int W, bool TRACK>
+static size_t sliced_bytes() {
+  return (sizeof(SlicedShared) + 15) / 16 * 16 + (TRACK ? sizeof(SlicedTrack<W>) : 0);
+}
+
+template <int W, bool VEC, bool TRACK>
+static int sliced_blocks_t() {
+  cudaFuncSetAttribute(graph_sliced_kernel<W, VEC, TRACK>,
+                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sliced_bytes<W, TRACK>());
+  static std::atomic<int> occ{0};
+  int o = occ.load(), dev = 0, sms = 152;
+  if (o == 0) {
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, graph_sliced_kernel<W, VEC, TRACK>,
+                                                  kSlicedTile, sliced_bytes<W, TRACK>());
+    occ = o > 0 ? o : 1;
+  }
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return (o > 0 ? o : 1) * sms;
+}
+
+template <int W, bool VEC, bool TRACK>
+static cudaError_t launch_sliced_t(const GraphJob* jobs, const Tile* tiles, int n_tiles,
+                                   uint32_t half, cudaStream_t st) {
+  const int blocks = sliced_blocks_t<W, VEC, TRACK>();
+  graph_sliced_kernel<W, VEC, TRACK><<<n_tiles < blocks ? n_tiles : blocks, kSlicedTile,
+                                       sliced_bytes<W, TRACK>(), st>>>(jobs, tiles, n_tiles, half);
+  return cudaGetLastError();
+}
+
+// shape: index in kSlicedShapes (words per thread, whole aligned rows)
+int graph_sliced_blocks(int shape, bool track) {
+  switch (shape) {
+    case 0: return track ? sliced_blocks_t<1, true, true>() : sliced_blocks_t<1, true, false>();
+    case 1: return track ? sliced_blocks_t<2, true, true>() : sliced_blocks_t<2, true, false>();
+    case 2: return track ? sliced_blocks_t<3, false, true>() : sliced_blocks_t<3, false, false>();
+    case 3: return track ? sliced_blocks_t<4, true, true>() : sliced_blocks_t<4, true, false>();
+    default: return track ? sliced_blocks_t<4, false, true>() : sliced_blocks_t<4, false, false>();
+  }
+}
+
+cudaError_t launch_graph_sliced(int shape, bool track, const GraphJob* jobs, const Tile* tiles,
+                                int n_tiles, uint32_t half, cudaStream_t st) {
+  if (n_tiles <= 0) return cudaSuccess;
+  switch (shape) {
+    case 0:
+      return track ? launch_sliced_t<1, true, true>(jobs, tiles, n_tiles, half, st)
+                   : launch_sliced_t<1, true, false>(jobs, tiles, n_tiles, half, st);
+    case 1:
+      return track ? launch_sliced_t<2, true, true>(jobs, tiles, n_tiles, half, st)
+                   : launch_sliced_t<2, true, false>(jobs, tiles, n_tiles, half, st);
+    case 2:
+      return track ? launch_sliced_t<3, false, true>(jobs, tiles, n_tiles, half, st)
+                   : launch_sliced_t<3, false, false>(jobs, tiles, n_tiles, half, st);
+    case 3:
+      return track ? launch_sliced_t<4, true, true>(jobs, tiles, n_tiles, half, st)
+                   : launch_sliced_t<4, true, false>(jobs, tiles, n_tiles, half, st);
+    default:
+      return track ? launch_sliced_t<4, false, true>(jobs, tiles, n_tiles, half, st)
+                   : launch_sliced_t<4, false, false>(jobs, tiles, n_tiles, half, st);
+  }
+}
+
+}  // namespace shk

@@ -42,6 +42,10 @@ cudaError_t launch_lattice_init(int, int, const LatJob*, const Tile*, int, int, 
 cudaError_t launch_lattice_obs(int, int, const LatJob*, const Tile*, int, int, int, cudaStream_t);
 cudaError_t launch_graph_half(bool, const GraphJob*, const Tile*, int, uint32_t, int, int,
                               cudaStream_t);
+cudaError_t launch_graph_sliced(int, bool, const GraphJob*, const Tile*, int, uint32_t,
+                                cudaStream_t);
+int graph_sliced_blocks(int, bool);
+int graph_half_blocks();
 cudaError_t launch_graph_hub(bool, const GraphJob*, const HubItem*, const uint32_t*, int, uint32_t,
                              uint32_t*, uint32_t*, cudaStream_t);
 cudaError_t launch_graph_init(const GraphJob*, const Tile*, int, int, cudaStream_t);
@@ -139,8 +143,13 @@ struct Family {
   int enc = 0;   // lattice encoding; graph: 1 integer couplings, 0 real
   int wpt = 1;   // lattice: lane words per thread per tile (tile = 256 wpt words)
   int bps = 0;   // lattice: resident blocks per SM of the half step (0: as many as fit)
-  DevMem jobs, tiles;  // graph: multi-group jobs and (vertex, group) pair tiles (half steps)
+  DevMem jobs, tiles;  // graph: multi-group jobs
   int n_tiles = 0;
+  // graph half steps, by position in the step: tiles of the bit-sliced kernel by shape and of
+  // the general one (ranges of the tile list)
+  struct Range {
+    int first = 0, n = 0;
+  } stiles[2][shk::kSlicedShapes], gtiles[2];
   DevMem ojobs, otiles;  // graph: one job per group and vertex tiles (init, observables)
   int n_otiles = 0;
   // graph: chunks of the edge lists of vertices of degree above kHubDeg, one warp per
@@ -243,6 +252,9 @@ struct shaken_ctx {
   DevMem series_m, series_H;
   DevMem in_ptr, in_col, in_J, out_ptr, out_col, out_J, lam_dev;
   DevMem in_visit, out_visit;  // half-step visiting order: (x, first edge, degree, lambda_x)
+  uint32_t sliced_slots[2][2] = {{0, 0}, {0, 0}};  // graph: slots of the degree order (in, out)
+                                                   // whose vertices have at most 16, 32
+                                                   // threshold classes
   std::vector<uint32_t> hubs[2];  // graph: (x, first edge, end edge) of the vertices of degree
                                   // above kHubDeg, in-CSR [0] and out-CSR [1]
   DevMem band_xch, band_sync;  // banded runs: row exchange area and grid barrier
@@ -273,14 +285,15 @@ static void add_tiles(std::vector<Tile>& tiles, uint32_t job, uint64_t count, ui
   for (uint64_t w = 0; w < count; w += size) tiles.push_back(Tile{job, (uint32_t)w});
 }
 
-// Graph half-step tiles of one job, vertices in degree order: the tiles are listed in
-// the order k -> (k * s) mod N with s coprime to N near N (sqrt 5 - 1) / 2, so the
-// heavy tiles (the highest degrees, at the end of the order) spread evenly over the
-// contiguous tile ranges the blocks take instead of all falling to the last blocks.
-static void add_graph_tiles(std::vector<Tile>& tiles, uint32_t job, uint64_t count,
+// Graph half-step tiles of one job over the slots [first, last) of the degree order: the
+// tiles are listed in the order k -> (k * s) mod N with s coprime to N near
+// N (sqrt 5 - 1) / 2, so the heavy tiles (the highest degrees, at the end of the order)
+// spread evenly over the contiguous tile ranges the blocks take instead of all falling
+// to the last blocks.
+static void add_graph_tiles(std::vector<Tile>& tiles, uint32_t job, uint64_t first, uint64_t last,
                             uint32_t size) {
-  const uint64_t N = (count + size - 1) / size;
-  if (N == 0) return;
+  if (first >= last) return;
+  const uint64_t N = (last - first + size - 1) / size;
   uint64_t st = (uint64_t)((double)N * 0.6180339887498949);
   if (st == 0) st = 1;
   auto gcd = [](uint64_t a, uint64_t b) {
@@ -294,7 +307,93 @@ static void add_graph_tiles(std::vector<Tile>& tiles, uint32_t job, uint64_t cou
   while (gcd(st, N) != 1) ++st;
   uint64_t pos = 0;
   for (uint64_t k = 0; k < N; ++k, pos = (pos + st) % N)
-    tiles.push_back(Tile{job, (uint32_t)(pos * size)});
+    tiles.push_back(Tile{job, (uint32_t)(first + pos * size)});
+}
+
+// The bit-sliced kernel's tiles, listed job by job and heaviest degrees first, rearranged so
+// that the blocks -- each walks a contiguous range, [b T / g, (b + 1) T / g) of T tiles for
+// a grid of g -- take a job's tiles in turn: the first tile of every range the heaviest
+// ones, and so on.  The ranges then weigh the same, and at any time all blocks run the code
+// of about one degree (the kernel's four class widths together overflow the instruction
+// cache).
+static void deal_tiles(std::vector<Tile>& tiles, int grid) {
+  const uint64_t T = tiles.size(), g = std::min<uint64_t>(T, (uint64_t)grid);
+  std::vector<Tile> out(T);
+  auto first = [&](uint64_t b) { return b * T / g; };
+  for (uint64_t p0 = 0, p1 = 0; p0 < T; p0 = p1) {
+    while (p1 < T && tiles[p1].job == tiles[p0].job) ++p1;
+    uint64_t b0 = p0 * g / T, next = p0;
+    while (first(b0 + 1) <= p0) ++b0;
+    for (uint64_t k = 0; next < p1; ++k)
+      for (uint64_t b = b0; b < g && first(b) < p1; ++b) {
+        const uint64_t pos = std::max(first(b), p0) + k;
+        if (pos < std::min(first(b + 1), p1)) out[pos] = tiles[next++];
+      }
+  }
+  tiles.swap(out);
+}
+
+// Threads per vertex of the bit-sliced kernel (a power of two) for ng groups in a shape.
+static uint32_t sliced_threads(uint32_t ng, int shape) {
+  uint32_t gp = 1;
+  while (gp * (uint32_t)shk::kSlicedWords[shape] < ng) gp <<= 1;
+  return gp;
+}
+
+// Shape of the bit-sliced kernel for a job of ng groups (rows of G words) and n vertices.  A
+// thread costs about as much for what its words share (class masks, columns, addresses) as
+// for one word, so the cheapest shape minimises threads x (1 + words); a job that does not
+// fill the GPU takes fewer words per thread, down to one, as long as it stays within one
+// wave (it is bound by each thread's own chain).
+static int sliced_shape(uint32_t ng, uint32_t G, uint64_t n) {
+  const uint64_t wave = (uint64_t)shk::graph_sliced_blocks(3, false) * shk::kSlicedTile;
+  int best = 0;
+  uint64_t cost = ~0ull;
+  for (int k = 0; k < shk::kSlicedShapes; ++k) {
+    const uint32_t w = (uint32_t)shk::kSlicedWords[k];
+    if (shk::kSlicedVec[k] && G % w != 0) continue;
+    const uint64_t gp = sliced_threads(ng, k);
+    if (gp > (uint64_t)shk::kSlicedTile) continue;
+    if (n * gp <= wave) return k;
+    if (gp * (1 + w) < cost) {
+      cost = gp * (1 + w);
+      best = k;
+    }
+  }
+  return best;
+}
+
+// Whether the bit-sliced kernel decides a graph context's low-degree vertices in the half
+// step at position `half` of a step: +-1 couplings and one inverse temperature on all
+// replicas.  Its tracking sums count agreeing edges, so with fields the tracked half
+// step stays with the general kernel.
+static bool sliced_half(const shaken_ctx* c, uint32_t half) {
+  if (!c->integer || c->exact_always) return false;
+  if (c->hcd.anneal_len == 0)
+    for (double b : c->beta)
+      if (b != c->beta[0]) return false;
+  if (half == 0 && c->hcd.tracking && !c->hcd.record && (c->has_lambda || c->lam_c != 0.0))
+    return false;
+  return true;
+}
+
+// Slots of the degree order that the bit-sliced kernel takes in a half step (whole tiles
+// unless all of them); the general kernel takes the rest, vertices of more than 32 classes.
+// With one or two words per thread a 32-class tree costs more than the general kernel's
+// byte lookups, so there a job of which more than 5 % of the vertices need one stays with
+// the general kernel (ten steps of an Erdos-Renyi graph, n = 3e5, R = 32: mean degree 8,
+// q = 0.7, 11 %: 1150 against 1070 us; q = 1, 1 %: 627 against 994 us; mean degree 4,
+// q = 2.5, 0 %: 571 against 818 us; a line at 16 classes within the job costs a second
+// launch: q = 1 1045 us).  So does a job within one wave that both kernels would have to share.
+static uint64_t sliced_cut(const shaken_ctx* c, uint32_t half, const GraphJob& H, int shape,
+                           uint32_t stile) {
+  if (H.sGp > (uint32_t)shk::kSlicedTile || !sliced_half(c, half)) return 0;
+  const uint32_t* slots = c->sliced_slots[half ^ c->hcd.order];
+  uint64_t cut = slots[1];
+  const bool wave = (uint64_t)c->n * H.Gp <= (uint64_t)shk::graph_half_blocks() * kTile;
+  if (wave) return cut == (uint64_t)c->n ? cut : 0;
+  if (shk::kSlicedWords[shape] <= 2 && (double)slots[0] < 0.95 * (double)c->n) return 0;
+  return cut == (uint64_t)c->n ? cut : cut - cut % stile;
 }
 
 static void lattice_tiles(const std::vector<LatJob>& jobs, uint32_t size,
@@ -439,7 +538,8 @@ static shaken_status build_plan(Plan& P, cudaStream_t st) {
   std::vector<std::vector<GraphJob>> gjobs(2);  // 0 integer, 1 real: half-step jobs
   std::vector<std::vector<GraphJob>> ojobs(2);  // per-group jobs
   std::vector<std::vector<Tile>> otiles(2);
-  std::vector<std::vector<Tile>> tiles(5);
+  std::vector<std::vector<Tile>> tiles(3);
+  std::vector<Tile> gtiles[2][2], stiles[2][2][shk::kSlicedShapes];  // [family][half], [.][.][shape]
   std::vector<std::vector<HubItem>> hitems(2);    // per graph family: hub chunks
   std::vector<std::vector<uint32_t>> hunits(2);   // unit -> item
   std::vector<uint32_t> hrows(2, 0u), hdone(2, 0u);
@@ -515,8 +615,17 @@ static shaken_status build_plan(Plan& P, cudaStream_t st) {
         H.Gj = std::min<uint32_t>((uint32_t)kTile, ng - g0);
         H.Gp = 1;
         while (H.Gp < H.Gj) H.Gp <<= 1;
-        add_graph_tiles(tiles[3 + fi], (uint32_t)gjobs[fi].size(), (uint64_t)c->n,
-                        (uint32_t)kTile / H.Gp);
+        const int shape = sliced_shape(H.Gj, ng, (uint64_t)c->n);
+        H.sGp = sliced_threads(H.Gj, shape);
+        const uint32_t stile = (uint32_t)shk::kSlicedTile / std::min(H.sGp, (uint32_t)shk::kSlicedTile);
+        for (uint32_t half = 0; half < 2; ++half) {
+          const uint64_t cut = sliced_cut(c, half, H, shape, stile);
+          for (uint64_t w0 = (cut + stile - 1) / stile * stile; w0 > 0; w0 -= stile)
+            stiles[fi][half][shape].push_back(
+                Tile{(uint32_t)gjobs[fi].size(), (uint32_t)(w0 - stile)});
+          add_graph_tiles(gtiles[fi][half], (uint32_t)gjobs[fi].size(), cut, (uint64_t)c->n,
+                          (uint32_t)kTile / H.Gp);
+        }
         for (uint32_t dir = 0; dir < 2; ++dir) {
           const std::vector<uint32_t>& hv = c->hubs[dir];
           for (size_t k = 0; k + 2 < hv.size(); k += 3) {
@@ -578,8 +687,23 @@ static shaken_status build_plan(Plan& P, cudaStream_t st) {
     F->kind = 1;
     F->enc = fi == 0 ? 1 : 0;
     TRY(upload(F->jobs, gjobs[fi].data(), gjobs[fi].size() * sizeof(GraphJob), st));
-    TRY(upload(F->tiles, tiles[3 + fi].data(), tiles[3 + fi].size() * sizeof(Tile), st));
-    F->n_tiles = (int)tiles[3 + fi].size();
+    std::vector<Tile> all;
+    auto put = [&](const std::vector<Tile>& t) {
+      Family::Range r;
+      r.first = (int)all.size();
+      r.n = (int)t.size();
+      all.insert(all.end(), t.begin(), t.end());
+      return r;
+    };
+    for (int half = 0; half < 2; ++half) {
+      for (int k = 0; k < shk::kSlicedShapes; ++k) {
+        std::vector<Tile>& sl = stiles[fi][half][k];
+        if (!sl.empty()) deal_tiles(sl, shk::graph_sliced_blocks(k, half == 0));
+        F->stiles[half][k] = put(sl);
+      }
+      F->gtiles[half] = put(gtiles[fi][half]);
+    }
+    TRY(upload(F->tiles, all.data(), all.size() * sizeof(Tile), st));
     TRY(upload(F->ojobs, ojobs[fi].data(), ojobs[fi].size() * sizeof(GraphJob), st));
     TRY(upload(F->otiles, otiles[fi].data(), otiles[fi].size() * sizeof(Tile), st));
     F->n_otiles = (int)otiles[fi].size();
@@ -604,7 +728,7 @@ static shaken_status plan_step_launch(Plan& P, cudaStream_t st, uint64_t* nl,
   uint64_t count = 0;
   const bool timed = P.timing > 0 && !capturing && P.steps_issued % (uint64_t)P.timing == 0;
   if (!capturing) ++P.steps_issued;
-  bool obs_needed = false;
+  bool obs_needed = false, track = false;
   int ex = 0;
   for (shaken_ctx* c : P.members) {
     // multispin lattices track with the observables kernel; graphs fuse tracking
@@ -612,6 +736,7 @@ static shaken_status plan_step_launch(Plan& P, cudaStream_t st, uint64_t* nl,
     if (c->hcd.tracking && c->kind == SHAKEN_LATTICE && c->enc == SHAKEN_MULTISPIN)
       obs_needed = true;
     if (c->hcd.tracking && c->kind == SHAKEN_GRAPH && c->hcd.record) obs_needed = true;
+    if (c->hcd.tracking && c->kind == SHAKEN_GRAPH && !c->hcd.record) track = true;
     ex |= c->exact_always;
   }
   if (obs_needed) {
@@ -635,13 +760,26 @@ static shaken_status plan_step_launch(Plan& P, cudaStream_t st, uint64_t* nl,
         e1 = P.get_event();
         CU(cudaEventRecord(e0, st));
       }
-      if (F->kind == 0)
+      if (F->kind == 0) {
         CU(shk::launch_lattice_half(F->enc, F->wpt, F->jobs.as<LatJob>(), F->tiles.as<Tile>(),
                                     F->n_tiles, half, P.rng_counter, st, F->bps));
-      else
-        CU(shk::launch_graph_half(F->enc != 0, F->jobs.as<GraphJob>(), F->tiles.as<Tile>(),
-                                  F->n_tiles, half, ex, P.blocks_per_sm, st));
-      ++count;
+        ++count;
+      } else {
+        for (int k = 0; k < shk::kSlicedShapes; ++k) {
+          const Family::Range& r = F->stiles[half][k];
+          if (r.n == 0) continue;
+          CU(shk::launch_graph_sliced(k, track && half == 0, F->jobs.as<GraphJob>(),
+                                      F->tiles.as<Tile>() + r.first, r.n, half, st));
+          ++count;
+        }
+        const Family::Range& r = F->gtiles[half];
+        if (r.n > 0) {
+          CU(shk::launch_graph_half(F->enc != 0, F->jobs.as<GraphJob>(),
+                                    F->tiles.as<Tile>() + r.first, r.n, half, ex,
+                                    P.blocks_per_sm, st));
+          ++count;
+        }
+      }
       if (F->kind == 1 && F->n_hub_units > 0) {
         CU(shk::launch_graph_hub(F->enc != 0, F->jobs.as<GraphJob>(), F->hub_items.as<HubItem>(),
                                  F->hub_units.as<uint32_t>(), F->n_hub_units, half,
@@ -901,12 +1039,17 @@ static void build_graph_host(shaken_ctx* c, const shaken_problem* p, HostPrep& h
   csr(tail, head, hp.optr, hp.ocol, hp.oJ);
   // visiting order of each half step: vertices by increasing degree (counting sort,
   // stable), so a warp's words have nearly equal edge loops and take the same path
-  auto by_degree = [&](const std::vector<int32_t>& ptr, std::vector<uint32_t>& visit) {
+  // threshold classes: d + 2 with q = 1 (collapsed), else 2 d + 2
+  const size_t dlim[2] = {p->q == 1.0 ? 14u : 7u, p->q == 1.0 ? 30u : 15u};
+  auto by_degree = [&](const std::vector<int32_t>& ptr, std::vector<uint32_t>& visit,
+                       uint32_t (&sliced)[2]) {
     int32_t dmax = 0;
     for (int64_t x = 0; x < n; ++x) dmax = std::max(dmax, ptr[x + 1] - ptr[x]);
     std::vector<int64_t> start((size_t)dmax + 2, 0);
     for (int64_t x = 0; x < n; ++x) start[(size_t)(ptr[x + 1] - ptr[x]) + 1]++;
     for (size_t k = 1; k < start.size(); ++k) start[k] += start[k - 1];
+    for (int k = 0; k < 2; ++k)
+      sliced[k] = (uint32_t)(dlim[k] + 1 < start.size() ? start[dlim[k] + 1] : n);
     visit.assign((size_t)n * 4, 0u);
     for (int64_t x = 0; x < n; ++x) {
       const size_t sl = (size_t)start[(size_t)(ptr[x + 1] - ptr[x])]++;
@@ -919,8 +1062,8 @@ static void build_graph_host(shaken_ctx* c, const shaken_problem* p, HostPrep& h
       visit[4 * sl + 3] = lb;
     }
   };
-  by_degree(hp.iptr, hp.ivisit);
-  by_degree(hp.optr, hp.ovisit);
+  by_degree(hp.iptr, hp.ivisit, c->sliced_slots[0]);
+  by_degree(hp.optr, hp.ovisit, c->sliced_slots[1]);
   auto hubs = [&](const std::vector<int32_t>& ptr, std::vector<uint32_t>& out) {
     out.clear();
     for (int64_t x = 0; x < n; ++x)
@@ -1673,6 +1816,7 @@ shaken_status shaken_load(shaken_ctx* ctx, const void* buf, size_t len) {
   ctx->hcd.tracking = h.tracking;
   ctx->hcd.anneal_len = 0;
   ctx->solo.invalidate();
+  if (ctx->owner) ctx->owner->plan.invalidate();  // its plan routes by the tracking flag
   return push_cd(ctx);
 }
 
@@ -1710,6 +1854,8 @@ shaken_status shaken_sync(shaken_ctx* ctx) {
 shaken_status shaken_debug_exact_always(shaken_ctx* ctx, int on) {
   if (!ctx) return fail(SHAKEN_E_INVAL, "ctx is NULL");
   ctx->exact_always = on ? 1 : 0;
+  ctx->solo.invalidate();  // the plan routes by this flag
+  if (ctx->owner) ctx->owner->plan.invalidate();
   return SHAKEN_OK;
 }
 

@@ -30,6 +30,11 @@ constexpr uint32_t kPhW1 = 0xBB67AE85u;
 constexpr uint32_t kInitStep = 0xFFFFFFFFu;  // step index of the initial draw
 
 constexpr int kTile = 256;  // threads per block; graph tiles hold kTile vertices
+constexpr int kSlicedTile = 128;  // threads per block (and tile) of the bit-sliced graph kernel
+// Its shapes: group words per thread, and whether rows are whole aligned vectors of them.
+constexpr int kSlicedShapes = 5;
+constexpr int kSlicedWords[kSlicedShapes] = {1, 2, 3, 4, 4};
+constexpr bool kSlicedVec[kSlicedShapes] = {true, true, false, true, false};
 
 // ---------------------------------------------------------------- dependent launches
 // The kernels of a step (half steps, observables, epilogue) are launched with
@@ -326,6 +331,7 @@ struct GraphJob {
   uint32_t g0;             // first group of this job
   uint32_t Gj;             // groups of this job
   uint32_t Gp;             // threads per vertex in half-step tiles (power of two >= Gj)
+  uint32_t sGp;            // the same in the bit-sliced kernel (W groups per thread)
   uint32_t key0, key1;
   uint32_t integer;
 };
