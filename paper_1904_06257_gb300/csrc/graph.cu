@@ -1,6 +1,5 @@
 // graph.cu -- half-step kernels of the shaken dynamics on an arbitrary graph
-// G = (V, E) (Sec. 2 of arXiv:1904.06257), multispin over replicas, and the
-// graph observables.
+// G = (V, E) (Sec. 2 of arXiv:1904.06257), multispin over replicas.
 //
 // Half step 0 (P^{1->2}): h_x = sum_{y : (y -> x) in E^o} J_xy s_y + q s_x + lambda_x,
 // half step 1 (P^{2->1}): h_x = sum_{y : (x -> y) in E^o} J_xy s'_y + q s'_x + lambda_x
@@ -187,23 +186,6 @@ __device__ __forceinline__ uint32_t real_lanes(const float (&h)[32], uint32_t S,
     }
   }
   return res;
-}
-
-// Per-replica partial values v[0..31] of the 32 lanes of a warp -> lane k holds the
-// sum over the warp of v[k] in v[0] (each level halves the values a lane keeps).
-template <typename V>
-__device__ __forceinline__ V warp_transpose_sum(V (&v)[32], int lane) {
-#pragma unroll
-  for (int s = 16; s >= 1; s >>= 1) {
-    const bool up = (lane & s) != 0;
-#pragma unroll
-    for (int i = 0; i < s; ++i) {
-      const V send = up ? v[i] : v[i + s];
-      const V keep = up ? v[i + s] : v[i];
-      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, s);
-    }
-  }
-  return v[0];
 }
 
 // Sum over the chunk's edges [e0, e1) of word (., g), lane l taking edges e0 + l,
@@ -790,145 +772,6 @@ __global__ void __launch_bounds__(kTile) graph_init_kernel(const GraphJob* __res
   }
 }
 
-// Adds one bit per lane (x) to the bit-sliced counter p (planes 0 .. B - 1).
-__device__ __forceinline__ void bs_add(uint32_t (&p)[8], uint32_t x, int B) {
-#pragma unroll
-  for (int b = 0; b < 8; ++b) {
-    if (b < B) {
-      const uint32_t c = p[b] & x;
-      p[b] ^= x;
-      x = c;
-    }
-  }
-}
-
-// Sums over the CSR edges (x -> y) of the warp's 32 vertices (thread t: vertex x of
-// lane t), for lane k's replica: esum = sum of J_xy s_x s_y with s_y from Y, and (if
-// want_cut) cut = the number of those edges with s_x != s_y.  Integer couplings: per
-// thread, bit-sliced counters of the agreeing products (chunks of 255 edges), whose
-// planes are transposed across the warp; real couplings: per-replica float sums,
-// transposed once.  A thread's edges are read four at a time, the loads of the four
-// independent of one another.
-template <bool INTEGER>
-__device__ __forceinline__ void obs_edges(const int32_t* ptr, const uint32_t* col,
-                                          const float* Jr, const uint32_t* Y, uint32_t x,
-                                          bool act, uint32_t S, uint32_t G, uint32_t g,
-                                          bool want_cut, int lane, double& esum, double& cut) {
-  const int e0 = act ? ptr[x] : 0;
-  const int d = act ? ptr[x + 1] - e0 : 0;
-  const int dmax = __reduce_max_sync(0xffffffffu, d);
-  const int dsum = __reduce_add_sync(0xffffffffu, d);
-  long long cj = 0, ca = 0;
-  float fv[INTEGER ? 1 : 32];
-#pragma unroll
-  for (int k = 0; k < (INTEGER ? 1 : 32); ++k) fv[k] = 0.0f;
-  for (int base = 0; base < dmax; base += 252) {
-    const int B = 32 - __clz(min(dmax - base, 255));  // planes for counts up to the chunk
-    uint32_t pj[8], pa[8];
-#pragma unroll
-    for (int b = 0; b < 8; ++b) pj[b] = pa[b] = 0u;
-    const int hi = min(d, base + 252);
-    for (int e = base; e < hi; e += 4) {
-      uint32_t cv[4], w[4];
-      float Jv[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) cv[i] = e + i < hi ? __ldg(col + e0 + e + i) : 0u;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        w[i] = e + i < hi ? __ldg(Y + (size_t)(cv[i] & 0x7fffffffu) * G + g) : 0u;
-        if (!INTEGER) Jv[i] = e + i < hi ? __ldg(Jr + e0 + e + i) : 0.0f;
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if (e + i < hi) {
-          const uint32_t agree = ~(S ^ w[i]);
-          if constexpr (INTEGER) {
-            bs_add(pj, agree ^ (0u - (cv[i] >> 31)), B);
-          } else {
-#pragma unroll
-            for (int k = 0; k < 32; ++k) fv[k] += ((agree >> k) & 1u) ? Jv[i] : -Jv[i];
-          }
-          if (want_cut) bs_add(pa, agree, B);
-        }
-      }
-    }
-#pragma unroll
-    for (int b = 0; b < 8; ++b) {
-      if (b < B) {
-        if (INTEGER) cj += (long long)warp_column_count(pj[b], lane) << b;
-        if (want_cut) ca += (long long)warp_column_count(pa[b], lane) << b;
-      }
-    }
-  }
-  if constexpr (INTEGER)
-    esum = (double)(2 * cj - dsum);
-  else
-    esum = (double)warp_transpose_sum(fv, lane);
-  cut = want_cut ? (double)(dsum - ca) : 0.0;
-}
-
-// Observables of one group (per-group jobs, Gj = 1): thread t of a tile takes vertex
-// w0 + t; the sums over the warp's 32 vertices reach lane k (replica 32 g + k) by bit
-// transposes of the sigma words and of bit-sliced edge counters (integer sums) or by
-// transposing butterflies (float sums), and the block adds its warps once per tile.
-template <bool INTEGER>
-__global__ void __launch_bounds__(kTile) graph_obs_kernel(const GraphJob* __restrict__ jobs,
-                                                          const Tile* __restrict__ tiles,
-                                                          int n_tiles, int which, int full) {
-  __shared__ double red[kTile / 32][32][kNumSums];
-  pdl_enter();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int ti = blockIdx.x; ti < n_tiles; ti += gridDim.x) {
-    const Tile tl = tiles[ti];
-    const GraphJob& J = jobs[tl.job];
-    const uint32_t G = J.G, g = J.g0;
-    const uint32_t x = tl.w0 + (uint32_t)threadIdx.x;
-    const bool act = x < J.n;
-    const uint32_t am = act ? 0xffffffffu : 0u;
-    const uint32_t S = act ? J.A[(size_t)x * G + g] : 0u;
-    const uint32_t S2 = (act && full) ? J.B[(size_t)x * G + g] : 0u;
-    const float lam = act ? (J.lambda != nullptr ? J.lambda[x] : J.lambda_c) : 0.0f;
-    const int nact = __popc(__ballot_sync(0xffffffffu, act));
-    double acc[kNumSums];
-#pragma unroll
-    for (int q = 0; q < kNumSums; ++q) acc[q] = 0.0;
-    acc[kSumM] = (double)(2 * warp_column_count(S & am, lane) - nact);
-    {
-      float v[32];
-#pragma unroll
-      for (int k = 0; k < 32; ++k) v[k] = ((S >> k) & 1u) ? lam : -lam;
-      acc[kSumLS] = (double)warp_transpose_sum(v, lane);
-    }
-    obs_edges<INTEGER>(J.in_ptr, J.in_col, J.in_J, J.A, x, act, S, G, g, true, lane,
-                       acc[kSumE], acc[kSumCut]);
-    if (full) {
-      acc[kSumP2] = (double)(2 * warp_column_count(~(S ^ S2) & am, lane) - nact);
-      float v[32];
-#pragma unroll
-      for (int k = 0; k < 32; ++k) v[k] = ((S2 >> k) & 1u) ? lam : -lam;
-      acc[kSumLS2] = (double)warp_transpose_sum(v, lane);
-      double unused;
-      obs_edges<INTEGER>(J.out_ptr, J.out_col, J.out_J, J.B, x, act, S, G, g, false, lane,
-                         acc[kSumP1], unused);
-    }
-#pragma unroll
-    for (int q = 0; q < kNumSums; ++q) red[warp][lane][q] = acc[q];
-    __syncthreads();
-    if (threadIdx.x < 32) {
-      double* dst = (which ? J.obs : J.sums) + (size_t)(32u * g + threadIdx.x) * kNumSums;
-#pragma unroll
-      for (int q = 0; q < kNumSums; ++q) {
-        if (q == kSumM2) continue;
-        if (!full && (q == kSumP1 || q == kSumP2 || q == kSumLS2)) continue;
-        double s = 0.0;
-        for (int wv = 0; wv < kTile / 32; ++wv) s += red[wv][threadIdx.x][q];
-        if (s != 0.0) atomicAdd(dst + q, s);
-      }
-    }
-    __syncthreads();
-  }
-}
-
 static int grid_for(int n_tiles, int per_sm) {
   int dev = 0, sms = 152;
   cudaGetDevice(&dev);
@@ -993,17 +836,6 @@ cudaError_t launch_graph_init(const GraphJob* jobs, const Tile* tiles, int n_til
   if (n_tiles <= 0) return cudaSuccess;
   graph_init_kernel<<<grid_for(n_tiles, 8), kTile, 0, st>>>(jobs, tiles, n_tiles, kind);
   return cudaGetLastError();
-}
-
-cudaError_t launch_graph_obs(bool integer, const GraphJob* jobs, const Tile* tiles, int n_tiles,
-                             int which, int full, cudaStream_t st) {
-  if (n_tiles <= 0) return cudaSuccess;
-  const dim3 grid(grid_for(n_tiles, 4));
-  if (integer)
-    return launch_dependent(graph_obs_kernel<true>, grid, dim3(kTile), 0, st, jobs, tiles,
-                            n_tiles, which, full);
-  return launch_dependent(graph_obs_kernel<false>, grid, dim3(kTile), 0, st, jobs, tiles,
-                          n_tiles, which, full);
 }
 
 cudaError_t launch_graph_fields(const GraphJob* jobs, const Tile* tiles, int n_tiles, uint32_t half,

@@ -99,4 +99,41 @@ static __device__ __noinline__ bool decide_lane(uint32_t key0, uint32_t key1, ui
   return (unsigned long long)u < threshold_T(h, beta);
 }
 
+// Per-replica partial values v[0..31] of the 32 lanes of a warp -> lane k holds the
+// sum over the warp of v[k] in v[0] (each level halves the values a lane keeps).
+template <typename V>
+__device__ __forceinline__ V warp_transpose_sum(V (&v)[32], int lane) {
+#pragma unroll
+  for (int s = 16; s >= 1; s >>= 1) {
+    const bool up = (lane & s) != 0;
+#pragma unroll
+    for (int i = 0; i < s; ++i) {
+      const V send = up ? v[i] : v[i + s];
+      const V keep = up ? v[i + s] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, s);
+    }
+  }
+  return v[0];
+}
+
+// Lane k's column of the warp's 32 words (bit i = bit k of lane i's word): five butterfly
+// exchanges, as in warp_column_count.
+__device__ __forceinline__ uint32_t warp_column(uint32_t x, int lane) {
+  const uint32_t Hm[5] = {0xFFFF0000u, 0xFF00FF00u, 0xF0F0F0F0u, 0xCCCCCCCCu, 0xAAAAAAAAu};
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    const int j = 16 >> i;
+    const uint32_t p = __shfl_xor_sync(0xffffffffu, x, j);
+    const bool hi = (lane & j) != 0;
+    const uint32_t t = hi ? (p >> j) : (p << j);
+    const uint32_t M = hi ? ~Hm[i] : Hm[i];
+    x = (x & ~M) | (t & M);
+  }
+  return x;
+}
+
+__device__ __forceinline__ uint32_t maj3(uint32_t a, uint32_t b, uint32_t c) {
+  return (a & b) | (a & c) | (b & c);
+}
+
 }  // namespace shk

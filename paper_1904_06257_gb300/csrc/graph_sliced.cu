@@ -98,10 +98,6 @@ __device__ __forceinline__ void st_words(uint32_t* p, uint32_t last, const uint3
   }
 }
 
-__device__ __forceinline__ uint32_t maj3(uint32_t a, uint32_t b, uint32_t c) {
-  return (a & b) | (a & c) | (b & c);
-}
-
 // 0 or ~0: the sign bit of byte B of t, replicated over the word.
 template <int B>
 __device__ __forceinline__ uint32_t byte_sign(uint32_t t) {
@@ -459,21 +455,6 @@ __device__ __forceinline__ void sliced_decide(SlicedShared& sh, SlicedTrack<W>* 
       sliced_round(sh, q + qn, 32, lane);
     }
   } while (__any_sync(0xffffffffu, cu != 0u));
-}
-
-// Lane k's column of the warp's 32 words (bit i = bit k of lane i's word).
-__device__ __forceinline__ uint32_t warp_column(uint32_t x, int lane) {
-  const uint32_t Hm[5] = {0xFFFF0000u, 0xFF00FF00u, 0xF0F0F0F0u, 0xCCCCCCCCu, 0xAAAAAAAAu};
-#pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    const int j = 16 >> i;
-    const uint32_t p = __shfl_xor_sync(0xffffffffu, x, j);
-    const bool hi = (lane & j) != 0;
-    const uint32_t t = hi ? (p >> j) : (p << j);
-    const uint32_t M = hi ? ~Hm[i] : Hm[i];
-    x = (x & ~M) | (t & M);
-  }
-  return x;
 }
 
 // The warp's counter planes into the block's totals (or, for jobs of more groups than the

@@ -49,7 +49,9 @@ int graph_half_blocks();
 cudaError_t launch_graph_hub(bool, const GraphJob*, const HubItem*, const uint32_t*, int, uint32_t,
                              uint32_t*, uint32_t*, cudaStream_t);
 cudaError_t launch_graph_init(const GraphJob*, const Tile*, int, int, cudaStream_t);
-cudaError_t launch_graph_obs(bool, const GraphJob*, const Tile*, int, int, int, cudaStream_t);
+cudaError_t launch_graph_obs(const GraphJob*, const Tile*, int, const HubItem*, const uint32_t*, int,
+                             int, int, cudaStream_t);
+cudaError_t launch_graph_obs_group(bool, const GraphJob*, const Tile*, int, int, int, cudaStream_t);
 cudaError_t launch_graph_fields(const GraphJob*, const Tile*, int, uint32_t, float*,
                                 cudaStream_t);
 cudaError_t launch_epilogue(CtxDev* const*, int, cudaStream_t);
@@ -150,7 +152,10 @@ struct Family {
   struct Range {
     int first = 0, n = 0;
   } stiles[2][shk::kSlicedShapes], gtiles[2];
-  DevMem ojobs, otiles;  // graph: one job per group and vertex tiles (init, observables)
+  Range vtiles;         // graph observables, integer couplings: all vertices of the half-step jobs
+  bool fields = false;  // graph: some member has lambda != 0
+  DevMem ojobs, otiles;  // graph: one job per group and vertex tiles (init, observables with
+                         // fields or real couplings, field dump)
   int n_otiles = 0;
   // graph: chunks of the edge lists of vertices of degree above kHubDeg, one warp per
   // (chunk, group) unit; partial rows and finished-chunk counters of their words
@@ -539,7 +544,7 @@ static shaken_status build_plan(Plan& P, cudaStream_t st) {
   std::vector<std::vector<GraphJob>> ojobs(2);  // per-group jobs
   std::vector<std::vector<Tile>> otiles(2);
   std::vector<std::vector<Tile>> tiles(3);
-  std::vector<Tile> gtiles[2][2], stiles[2][2][shk::kSlicedShapes];  // [family][half], [.][.][shape]
+  std::vector<Tile> gtiles[2][2], vtiles[2], stiles[2][2][shk::kSlicedShapes];  // [family][half], [.][.][shape]
   std::vector<std::vector<HubItem>> hitems(2);    // per graph family: hub chunks
   std::vector<std::vector<uint32_t>> hunits(2);   // unit -> item
   std::vector<uint32_t> hrows(2, 0u), hdone(2, 0u);
@@ -626,6 +631,9 @@ static shaken_status build_plan(Plan& P, cudaStream_t st) {
           add_graph_tiles(gtiles[fi][half], (uint32_t)gjobs[fi].size(), cut, (uint64_t)c->n,
                           (uint32_t)kTile / H.Gp);
         }
+        if (c->integer)
+          add_graph_tiles(vtiles[fi], (uint32_t)gjobs[fi].size(), 0, (uint64_t)c->n,
+                          (uint32_t)kTile / H.Gp);
         for (uint32_t dir = 0; dir < 2; ++dir) {
           const std::vector<uint32_t>& hv = c->hubs[dir];
           for (size_t k = 0; k + 2 < hv.size(); k += 3) {
@@ -703,6 +711,10 @@ static shaken_status build_plan(Plan& P, cudaStream_t st) {
       }
       F->gtiles[half] = put(gtiles[fi][half]);
     }
+    F->vtiles = put(vtiles[fi]);
+    for (const shaken_ctx* c : P.members)
+      if (c->kind == SHAKEN_GRAPH && c->integer == (fi == 0) && (c->has_lambda || c->lam_c != 0.0))
+        F->fields = true;
     TRY(upload(F->tiles, all.data(), all.size() * sizeof(Tile), st));
     TRY(upload(F->ojobs, ojobs[fi].data(), ojobs[fi].size() * sizeof(GraphJob), st));
     TRY(upload(F->otiles, otiles[fi].data(), otiles[fi].size() * sizeof(Tile), st));
@@ -720,6 +732,22 @@ static shaken_status build_plan(Plan& P, cudaStream_t st) {
   TRY(upload(P.ctxlist, cds.data(), cds.size() * sizeof(CtxDev*), st));
   P.n_ctx = (int)cds.size();
   P.dirty = false;
+  return SHAKEN_OK;
+}
+
+// Observables launches of a graph family (which, full: see the kernels).
+static shaken_status graph_obs(const Family& F, int which, int full, cudaStream_t st,
+                               uint64_t* launches) {
+  if (F.enc != 0) {
+    CU(shk::launch_graph_obs(F.jobs.as<GraphJob>(), F.tiles.as<Tile>() + F.vtiles.first,
+                             F.vtiles.n, F.hub_items.as<HubItem>(), F.hub_units.as<uint32_t>(),
+                             F.n_hub_units, which, full, st));
+    *launches += F.n_hub_units > 0 ? 2 : 1;
+    if (!F.fields) return SHAKEN_OK;
+  }
+  CU(shk::launch_graph_obs_group(F.enc != 0, F.ojobs.as<GraphJob>(), F.otiles.as<Tile>(),
+                                 F.n_otiles, which, full, st));
+  ++*launches;
   return SHAKEN_OK;
 }
 
@@ -746,9 +774,7 @@ static shaken_status plan_step_launch(Plan& P, cudaStream_t st, uint64_t* nl,
                                    F->n_tiles, 0, 0, st));
         ++count;
       } else if (F->kind == 1) {
-        CU(shk::launch_graph_obs(F->enc != 0, F->ojobs.as<GraphJob>(), F->otiles.as<Tile>(),
-                                 F->n_otiles, 0, 0, st));
-        ++count;
+        TRY(graph_obs(*F, 0, 0, st, &count));
       }
     }
   }
@@ -1524,9 +1550,8 @@ static shaken_status obs_launch(Plan& P, cudaStream_t st, uint64_t* launches) {
       CU(shk::launch_lattice_obs(F->enc, F->wpt, F->jobs.as<LatJob>(), F->tiles.as<Tile>(),
                                  F->n_tiles, 1, 1, st));
     else
-      CU(shk::launch_graph_obs(F->enc != 0, F->ojobs.as<GraphJob>(), F->otiles.as<Tile>(),
-                               F->n_otiles, 1, 1, st));
-    ++*launches;
+      TRY(graph_obs(*F, 1, 1, st, launches));
+    if (F->kind == 0) ++*launches;
   }
   return SHAKEN_OK;
 }
