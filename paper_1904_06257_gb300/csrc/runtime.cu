@@ -60,6 +60,8 @@ cudaError_t launch_member_copy(int, const shk::MemberDev*, int, void*, unsigned 
 bool lattice_band_shape(int, uint32_t, uint32_t, int*, size_t*);
 cudaError_t launch_lattice_band(int, const LatJob*, int, size_t, uint64_t*, BandSync*, uint32_t,
                                 uint32_t, cudaStream_t);
+int lattice_cluster_shape(uint32_t, int, double*);
+cudaError_t launch_lattice_cluster(const LatJob*, int, uint32_t, int, uint32_t, uint32_t, cudaStream_t);
 cudaError_t launch_lattice_resident(int, const LatJob*, int, uint32_t, uint32_t, uint32_t,
                                     cudaStream_t);
 cudaError_t launch_philox(uint64_t, const uint32_t*, uint32_t*, int64_t, cudaStream_t);
@@ -263,6 +265,8 @@ struct shaken_ctx {
   std::vector<uint32_t> hubs[2];  // graph: (x, first edge, end edge) of the vertices of degree
                                   // above kHubDeg, in-CSR [0] and out-CSR [1]
   DevMem band_xch, band_sync;  // banded runs: row exchange area and grid barrier
+  int cluster = -1;            // MULTISPIN whole runs: blocks per cluster (0: no; -1: not known yet)
+  double cluster_us = 0.0;     // and the time of a step that way
   bool band_stall = false;     // diagnostics: the next banded run's barrier never completes
   int band_hurry = -1;         // diagnostics: block that gives up the next run's last wait at once
   CtxDev hcd{};
@@ -1296,29 +1300,50 @@ static shaken_status check_steps(shaken_ctx* c, uint64_t n) {
   return SHAKEN_OK;
 }
 
-// Small lattices run whole chunks of steps inside one launch, one block per
-// replica (or multispin group), the state in shared memory.
+// Small INT8 / PACKED lattices run whole chunks of steps inside one launch, one block per
+// replica, the state in shared memory.
 static bool resident_eligible(const shaken_ctx* c, uint64_t n_steps) {
-  if (c->kind != SHAKEN_LATTICE || c->owner || n_steps < 4) return false;
-  const uint64_t words = c->enc == SHAKEN_MULTISPIN ? (uint64_t)c->L * c->L
-                                                    : (uint64_t)c->L * c->L / 32;
-  if (words > 4096) return false;
-  if (c->enc == SHAKEN_MULTISPIN && (c->hcd.tracking || c->hcd.record)) return false;
-  return true;
+  if (c->kind != SHAKEN_LATTICE || c->owner || n_steps < 4 || c->enc == SHAKEN_MULTISPIN)
+    return false;
+  return (uint64_t)c->L * c->L / 32 <= 4096;
+}
+
+// Small MULTISPIN lattices: one thread-block cluster per group of 32 replicas, where that takes
+// less time per step than the kernels of a step on the whole GPU.  Both in microseconds per
+// step, fitted to sides 32 .. 256 and 1 .. 64 groups: a half step in a cluster is its chain
+// and 1.9 ns per word of a block (shk::lattice_cluster_shape), with tracking 1 us more; the kernels
+// take 8.5 us and 22 ns per 1000 words, with tracking 10 us and 14 ns more.  Measured on both
+// sides of the line, 100 steps: L = 192, 1 group 1180 (cluster) against 1000 us, 4
+// groups 1185 against 1455; tracked 4 groups 1422 against 2523.
+static bool cluster_eligible(shaken_ctx* c, uint64_t n_steps) {
+  if (c->kind != SHAKEN_LATTICE || c->owner || n_steps < 4 || c->enc != SHAKEN_MULTISPIN)
+    return false;
+  const int groups = c->R / 32;
+  if (c->cluster < 0)
+    c->cluster = shk::lattice_cluster_shape((uint32_t)c->L, groups, &c->cluster_us);
+  if (c->cluster == 0) return false;
+  const double words = (double)c->L * (double)c->L * groups;
+  const bool tr = c->hcd.tracking != 0;
+  return c->cluster_us + (tr ? 1.0 : 0.0) < (tr ? 18.5 : 8.5) + (tr ? 3.6e-5 : 2.2e-5) * words;
 }
 
 static shaken_status run_resident(shaken_ctx* c, uint64_t n_steps) {
   cudaStream_t st = c->stream;
   if (c->solo.dirty) TRY(build_plan(c->solo, st));
   const Family& F = *c->solo.fams[0];
-  const int n_jobs = c->enc == SHAKEN_MULTISPIN ? c->R / 32 : c->R;
-  const uint32_t words = c->enc == SHAKEN_MULTISPIN ? (uint32_t)(c->L * c->L)
-                                                    : (uint32_t)(c->L * c->L / 32);
+  const bool cluster = c->enc == SHAKEN_MULTISPIN;
+  const int n_jobs = cluster ? c->R / 32 : c->R;
+  const uint32_t words = (uint32_t)(c->L * c->L / 32);
   uint64_t done = 0;
   while (done < n_steps) {
     const uint64_t chunk = std::min<uint64_t>(n_steps - done, 1u << 16);
-    CU(shk::launch_lattice_resident(F.enc, F.jobs.as<LatJob>(), n_jobs, words,
-                                    (uint32_t)(c->host_step + done), (uint32_t)chunk, st));
+    const uint32_t t = (uint32_t)(c->host_step + done);
+    if (cluster)
+      CU(shk::launch_lattice_cluster(F.jobs.as<LatJob>(), n_jobs, (uint32_t)c->L, c->cluster, t,
+                                     (uint32_t)chunk, st));
+    else
+      CU(shk::launch_lattice_resident(F.enc, F.jobs.as<LatJob>(), n_jobs, words, t,
+                                      (uint32_t)chunk, st));
     c->launches++;
     done += chunk;
   }
@@ -1378,7 +1403,8 @@ static shaken_status run_band(shaken_ctx* c, uint64_t n_steps, int grid, size_t 
 }
 
 static shaken_status solo_run(shaken_ctx* ctx, uint64_t n_steps) {
-  if (resident_eligible(ctx, n_steps)) return run_resident(ctx, n_steps);
+  if (resident_eligible(ctx, n_steps) || cluster_eligible(ctx, n_steps))
+    return run_resident(ctx, n_steps);
   int grid = 0;
   size_t smem = 0;
   if (band_eligible(ctx, n_steps, &grid, &smem)) return run_band(ctx, n_steps, grid, smem);
