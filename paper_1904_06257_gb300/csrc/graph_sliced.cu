@@ -27,7 +27,7 @@
 #include <atomic>
 #include <cstdint>
 
-#include "graph_device.cuh"
+#include "graph_planes.cuh"
 #include "shaken_internal.cuh"
 
 namespace shk {
@@ -98,87 +98,6 @@ __device__ __forceinline__ void st_words(uint32_t* p, uint32_t last, const uint3
   }
 }
 
-// 0 or ~0: the sign bit of byte B of t, replicated over the word.
-template <int B>
-__device__ __forceinline__ uint32_t byte_sign(uint32_t t) {
-  uint32_t r;
-  asm("prmt.b32 %0, %1, 0, %2;" : "=r"(r) : "r"(t), "n"(0x8888 + 0x1111 * B));
-  return r;
-}
-
-// Selects leaf idx of 2^NB leaves given by the sign bits of the bytes of tb[0 .. 2^NB / 4),
-// for each of W words with idx planes I[b][.].
-template <int NB, int W>
-__device__ __forceinline__ void mux_tree(const uint32_t* tb, const uint32_t (*I)[W],
-                                         uint32_t (&q)[W]) {
-  if constexpr (NB == 2) {
-    const uint32_t m0 = byte_sign<0>(tb[0]), m1 = byte_sign<1>(tb[0]), m2 = byte_sign<2>(tb[0]),
-                   m3 = byte_sign<3>(tb[0]);
-#pragma unroll
-    for (int j = 0; j < W; ++j) {
-      const uint32_t lo = (I[0][j] & m1) | (~I[0][j] & m0);
-      const uint32_t hi = (I[0][j] & m3) | (~I[0][j] & m2);
-      q[j] = (I[1][j] & hi) | (~I[1][j] & lo);
-    }
-  } else {
-    uint32_t lo[W], hi[W];
-    mux_tree<NB - 1, W>(tb, I, lo);
-    mux_tree<NB - 1, W>(tb + (1 << NB) / 8, I, hi);
-#pragma unroll
-    for (int j = 0; j < W; ++j) q[j] = (I[NB - 1][j] & hi[j]) | (~I[NB - 1][j] & lo[j]);
-  }
-}
-
-// What a thread knows about its vertex and words.
-template <int W>
-struct SlicedWord {
-  uint32_t x, go, d, slot;  // vertex, first group of the thread within the job, degree, slot
-  uint32_t last;            // words of the thread beyond the first
-  int p0;
-  bool valid, collapse;
-  uint32_t F;        // frozen mask
-  uint32_t vamb;     // classes of uncertain top byte
-  uint32_t h01[W], l01[W];  // Philox: halves of M0 * u0 of the thread's groups
-  uint32_t c3base;   // update type
-  uint32_t u1;
-};
-
-// The Philox call of planes 4 call .. 4 call + 3 for the thread's W groups (counter words
-// (x, g, t, typ + 2 call)): x, t and the call are common to the words, so round 0 and
-// half of rounds 1 and 2 are computed once (ph_call_shared shares over x instead).
-template <int W>
-__device__ __forceinline__ void sliced_call(const uint2* key, const SlicedWord<W>& w,
-                                            uint32_t c3, uint32_t (&o)[4][W]) {
-  const unsigned long long p0 = (unsigned long long)kPhM0 * w.x;
-  const unsigned long long p1 =
-      (unsigned long long)kPhM1 * ((uint32_t)(p0 >> 32) ^ c3 ^ key[0].y);
-  const uint32_t a0 = (uint32_t)(p1 >> 32) ^ w.u1 ^ key[1].x;
-  const uint32_t a1 = (uint32_t)p1;
-  const unsigned long long q0 = (unsigned long long)kPhM0 * a0;
-#pragma unroll
-  for (int j = 0; j < W; ++j) {
-    const uint32_t c2 = w.h01[j] ^ (uint32_t)p0 ^ key[1].y;
-    const unsigned long long q1 = (unsigned long long)kPhM1 * c2;
-    o[0][j] = (uint32_t)(q1 >> 32) ^ a1 ^ key[2].x;
-    o[1][j] = (uint32_t)q1;
-    o[2][j] = (uint32_t)(q0 >> 32) ^ w.l01[j] ^ key[2].y;
-    o[3][j] = (uint32_t)q0;
-  }
-#pragma unroll
-  for (int r = 3; r < 10; ++r) {
-    const uint2 k = key[r];
-#pragma unroll
-    for (int j = 0; j < W; ++j) {
-      const unsigned long long s0 = (unsigned long long)kPhM0 * o[0][j];
-      const unsigned long long s1 = (unsigned long long)kPhM1 * o[2][j];
-      o[0][j] = (uint32_t)(s1 >> 32) ^ o[1][j] ^ k.x;
-      o[2][j] = (uint32_t)(s0 >> 32) ^ o[3][j] ^ k.y;
-      o[1][j] = (uint32_t)s1;
-      o[3][j] = (uint32_t)s0;
-    }
-  }
-}
-
 // Up to 32 entries of the warp's queue: lane i decides entry i (i < cnt) and sets its bit in
 // the stored word if it is +1.  Entry: (slot, k | idx << 5 | go << 10 | byte << 18 | amb << 26).
 __device__ __noinline__ void sliced_round(const SlicedShared& sh, const uint2* q, int cnt,
@@ -190,56 +109,12 @@ __device__ __noinline__ void sliced_round(const SlicedShared& sh, const uint2* q
     const uint4 vi = __ldg((sh.typ == 0u ? J.in_visit : J.out_visit) + e.x);
     const int k = (int)(e.y & 31u);
     const uint32_t idx = (e.y >> 5) & 31u, g = J.g0 + ((e.y >> 10) & 255u);
-    const bool collapse = sh.collapse != 0u;
-    const int a = (int)(collapse ? idx : idx >> 1), sig = collapse ? 0 : (int)(idx & 1u);
-    const int d = (int)vi.z;
-    const float lam = __uint_as_float(vi.w), qf = (float)J.q;
-    const float lmd = __fadd_rn(lam, -(float)d);
-    const float bp = __fadd_rn(lmd, qf), bm = __fadd_rn(lmd, -qf);
-    const float B = (float)d + fabsf(qf) + fabsf(lam) + 1.0f;
-    uint32_t u8 = (e.y >> 18) & 0xFFu;
-    if ((e.y >> 26) & 1u) {  // class of uncertain top byte: the draw's own
-      const PhKey K = ph_key(J.key0, J.key1);
-      const uint4 c0 = ph_call(K, vi.x, g, sh.t, sh.typ), c1 = ph_call(K, vi.x, g, sh.t, sh.typ + 2u);
-      u8 = lane_byte(c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w, k);
-    }
-    if (decide_lane(J.key0, J.key1, vi.x, g, sh.t, sh.typ, k, u8, a, d, sig, bp, bm, J.q, lam,
-                    sh.kb, fabsf(sh.kb) * B, sh.beta, false))
+    if (sliced_lane(J.key0, J.key1, vi.x, g, sh.t, sh.typ, J.q, sh.collapse != 0u, sh.kb, sh.beta,
+                    (int)vi.z, __uint_as_float(vi.w), k, idx, (e.y >> 18) & 0xFFu,
+                    ((e.y >> 26) & 1u) != 0u))
       atomicOr(sh.dst + (size_t)vi.x * J.G + g, 1u << k);
   }
   __syncwarp();
-}
-
-constexpr int kIdx = 5;  // planes of a class index (at most 32 classes)
-
-// Planes 4 call + 3 .. 4 call (least significant first) of the draws o against the
-// thresholds of vertices with at most 2^NB classes.  The call's class bits are the upper
-// (call 1: planes 7..4) or lower four of the bit-reversed bytes.
-template <int NB, int W>
-__device__ __forceinline__ void sliced_planes(const uint8_t* tbv, int call,
-                                              const uint32_t (&I)[kIdx][W], uint32_t (&o)[4][W],
-                                              uint32_t (&lt)[W], uint32_t (&eq)[W]) {
-  constexpr int NW = (1 << NB) / 4;
-  uint32_t tb[NW];
-#pragma unroll
-  for (int k = 0; k < NW; ++k)
-    tb[k] = reinterpret_cast<const uint32_t*>(tbv)[k] << (call != 0 ? 0 : 4);
-  auto plane = [&]() {
-    uint32_t Q[W];
-    mux_tree<NB, W>(tb, I, Q);
-#pragma unroll
-    for (int k = 0; k < NW; ++k) tb[k] <<= 1;
-#pragma unroll
-    for (int j = 0; j < W; ++j) {
-      lt[j] = maj3(~o[3][j], Q[j], lt[j]);
-      eq[j] &= ~(o[3][j] ^ Q[j]);
-      o[3][j] = o[2][j];
-      o[2][j] = o[1][j];
-      o[1][j] = o[0][j];
-    }
-  };
-#pragma unroll 1
-  for (int i = 0; i < 4; ++i) plane();  // a loop, for the instruction cache
 }
 
 // Decisions of the warp's vertices (one tile row); ncls: the most classes among them.
@@ -492,27 +367,6 @@ __device__ __noinline__ void sliced_flush(SlicedShared& sh, SlicedTrack<W>* tr, 
   }
 }
 
-// Class i of a vertex of degree d and field lam: its top byte into tbv[i] (bit-reversed);
-// 1 if the bounds do not fix it.
-__device__ __forceinline__ uint32_t sliced_class(const SlicedShared& sh, uint32_t i, uint32_t d,
-                                                 float lam, uint8_t* tbv) {
-  const uint32_t a = sh.collapse ? i : i >> 1;
-  const bool up = !sh.collapse && (i & 1u) != 0u;
-  const float qf = (float)sh.J.q, fd = (float)d;
-  const float h0 = __fadd_rn(__fadd_rn(lam, -fd), up ? qf : -qf);  // h = 2a + (lambda - d +- q)
-  const float hf = fmaf(2.0f, (float)a, h0);
-  float lo, hi;
-  t_bounds(hf, sh.kb, fabsf(sh.kb) * (fd + fabsf(qf) + fabsf(lam) + 1.0f), lo, hi);
-  uint32_t bl = top_byte(lo), bh = top_byte(hi);
-  // a field of exactly 0 has T = 2^31; with lambda = 0 and an integer q the fp32 field is
-  // exact
-  if (hf == 0.0f &&
-      (lam == 0.0f ? sh.qint != 0u : field_is_zero(2 * (int)a - (int)d, up, sh.J.q, lam)))
-    bl = bh = 0x80u;
-  tbv[i] = (uint8_t)(__brev(bh) >> 24);
-  return bl != bh ? 1u : 0u;
-}
-
 template <int W, bool VEC, bool TRACK>
 __global__ void __launch_bounds__(kSlicedTile, 4) graph_sliced_kernel(
     const GraphJob* __restrict__ jobs, const Tile* __restrict__ tiles, int n_tiles,
@@ -606,7 +460,8 @@ __global__ void __launch_bounds__(kSlicedTile, 4) graph_sliced_kernel(
         const uint32_t ncls = sh.collapse ? d + 2u : 2u * d + 2u;
         uint32_t mine = 0u;
         for (uint32_t i = (uint32_t)tid & 3u; i < ncls && i < 32u; i += 4u)
-          mine |= sliced_class(sh, i, d, J.lambda_c, &sh.tb[0][0][0] + 32u * d) << i;
+          mine |= sliced_class(J.q, sh.collapse != 0u, sh.qint != 0u, sh.kb, i, d, J.lambda_c,
+                               &sh.tb[0][0][0] + 32u * d) << i;
         mine |= __shfl_xor_sync(0xffffffffu, mine, 1);
         mine |= __shfl_xor_sync(0xffffffffu, mine, 2);
         if ((tid & 3) == 0) sh.amb[d] = mine;
@@ -654,7 +509,7 @@ __global__ void __launch_bounds__(kSlicedTile, 4) graph_sliced_kernel(
       uint8_t* own = sh.tb[warp][(uint32_t)lane / sw];
       uint32_t mine = 0u;
       for (uint32_t i = gs; i < ncls; i += sw)
-        mine |= sliced_class(sh, i, w.d, lam, own) << i;
+        mine |= sliced_class(J.q, w.collapse, sh.qint != 0u, sh.kb, i, w.d, lam, own) << i;
       for (uint32_t s = 1u; s < sw; s <<= 1) mine |= __shfl_xor_sync(0xffffffffu, mine, s);
       w.vamb = mine;
       tbv = own;

@@ -45,6 +45,9 @@ cudaError_t launch_graph_half(bool, const GraphJob*, const Tile*, int, uint32_t,
 cudaError_t launch_graph_sliced(int, bool, const GraphJob*, const Tile*, int, uint32_t,
                                 cudaStream_t);
 int graph_sliced_blocks(int, bool);
+int graph_cluster_shape(uint32_t, uint64_t, int, double*);
+cudaError_t launch_graph_cluster(const GraphJob*, int, uint32_t, uint64_t, int, CtxDev* const*, int,
+                                 uint32_t, cudaStream_t);
 int graph_half_blocks();
 cudaError_t launch_graph_hub(bool, const GraphJob*, const HubItem*, const uint32_t*, int, uint32_t,
                              uint32_t*, uint32_t*, cudaStream_t);
@@ -170,6 +173,12 @@ struct Plan {
   std::vector<std::unique_ptr<Family>> fams;
   DevMem ctxlist;
   int n_ctx = 0;
+  // graph members stepped in whole runs, one cluster of cl_blocks blocks per group (cl_clusters
+  // of them, cl_n_ctx members of at most cl_n vertices and cl_m edges); the others: ctxlist
+  DevMem cl_jobs, cl_ctx;
+  int cl_clusters = 0, cl_blocks = 0, cl_n_ctx = 0;
+  uint32_t cl_n = 0;
+  uint64_t cl_m = 0;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
   int graph_steps = 0;
@@ -540,9 +549,50 @@ static shaken_status choose_lattice_shape(const Plan& P, int enc, const std::vec
   return SHAKEN_OK;
 }
 
+// Whether the graph members of a plan are stepped in whole runs by graph_cluster_kernel: +-1
+// couplings, one lambda, every vertex and half step within the bit-sliced kernel, and less
+// time per step than the half-step kernels and the epilogue, which take 18 us (a small job's three
+// chains of launches and dependent loads) and 50 ns per 1000 words.  Measured on both sides of the
+// line, 100 tracked steps of mean degree 8: n = 4000, one group 1790 (cluster) against 2470 us,
+// eight groups 1890 against 2680; n = 16000, one group 3330 against 2540.  (With a lambda per
+// vertex the class bytes of a thread's vertex are its own work: 2350 against 1810 us at
+// n = 4000.)  Sets the plan's cluster size.
+static void choose_clusters(Plan& P) {
+  P.cl_clusters = P.cl_blocks = P.cl_n_ctx = 0;
+  P.cl_n = 0;
+  P.cl_m = 0;
+  if (P.timing > 0) return;  // timed runs bracket the half-step launches
+  double words = 0.0;
+  int clusters = 0, members = 0;
+  uint32_t most = 0;
+  uint64_t edges = 0;
+  for (const shaken_ctx* c : P.members) {
+    if (c->kind != SHAKEN_GRAPH) continue;
+    if (c->n > (int64_t)1 << 20 || !sliced_half(c, 0) || !sliced_half(c, 1) ||
+        c->sliced_slots[0][1] != (uint32_t)c->n || c->sliced_slots[1][1] != (uint32_t)c->n)
+      return;
+    if (c->has_lambda || (c->hcd.tracking && c->lam_c != 0.0)) return;
+    ++members;
+    clusters += c->R / 32;
+    words += (double)c->n * (c->R / 32);
+    most = std::max(most, (uint32_t)c->n);
+    edges = std::max(edges, (uint64_t)c->m);
+  }
+  if (members == 0 || clusters > 1024) return;
+  double us = 0.0;
+  const int blocks = shk::graph_cluster_shape(most, edges, clusters, &us);
+  if (blocks == 0 || us >= 18.0 + 5e-5 * words) return;
+  P.cl_clusters = clusters;
+  P.cl_blocks = blocks;
+  P.cl_n_ctx = members;
+  P.cl_n = most;
+  P.cl_m = edges;
+}
+
 static shaken_status build_plan(Plan& P, cudaStream_t st) {
   P.fams.clear();
   P.drop_graph();
+  choose_clusters(P);
   std::vector<std::vector<LatJob>> ljobs(3);
   std::vector<std::vector<GraphJob>> gjobs(2);  // 0 integer, 1 real: half-step jobs
   std::vector<std::vector<GraphJob>> ojobs(2);  // per-group jobs
@@ -552,10 +602,11 @@ static shaken_status build_plan(Plan& P, cudaStream_t st) {
   std::vector<std::vector<HubItem>> hitems(2);    // per graph family: hub chunks
   std::vector<std::vector<uint32_t>> hunits(2);   // unit -> item
   std::vector<uint32_t> hrows(2, 0u), hdone(2, 0u);
-  std::vector<CtxDev*> cds;
+  std::vector<CtxDev*> cds, cl_cds;
   for (shaken_ctx* c : P.members) {
     CtxDev* cdp = c->cd.as<CtxDev>();
-    cds.push_back(cdp);
+    const bool in_cluster = c->kind == SHAKEN_GRAPH && P.cl_clusters > 0;
+    (in_cluster ? cl_cds : cds).push_back(cdp);
     const uint32_t key0 = (uint32_t)(c->seed & 0xffffffffu), key1 = (uint32_t)(c->seed >> 32);
     if (c->kind == SHAKEN_LATTICE) {
       const int e = c->enc;
@@ -627,7 +678,7 @@ static shaken_status build_plan(Plan& P, cudaStream_t st) {
         const int shape = sliced_shape(H.Gj, ng, (uint64_t)c->n);
         H.sGp = sliced_threads(H.Gj, shape);
         const uint32_t stile = (uint32_t)shk::kSlicedTile / std::min(H.sGp, (uint32_t)shk::kSlicedTile);
-        for (uint32_t half = 0; half < 2; ++half) {
+        for (uint32_t half = 0; half < 2 && !in_cluster; ++half) {
           const uint64_t cut = sliced_cut(c, half, H, shape, stile);
           for (uint64_t w0 = (cut + stile - 1) / stile * stile; w0 > 0; w0 -= stile)
             stiles[fi][half][shape].push_back(
@@ -733,8 +784,12 @@ static shaken_status build_plan(Plan& P, cudaStream_t st) {
     }
     P.fams.push_back(std::move(F));
   }
-  TRY(upload(P.ctxlist, cds.data(), cds.size() * sizeof(CtxDev*), st));
+  if (!cds.empty()) TRY(upload(P.ctxlist, cds.data(), cds.size() * sizeof(CtxDev*), st));
   P.n_ctx = (int)cds.size();
+  if (P.cl_clusters > 0) {
+    TRY(upload(P.cl_jobs, ojobs[0].data(), ojobs[0].size() * sizeof(GraphJob), st));
+    TRY(upload(P.cl_ctx, cl_cds.data(), cl_cds.size() * sizeof(CtxDev*), st));
+  }
   P.dirty = false;
   return SHAKEN_OK;
 }
@@ -760,26 +815,25 @@ static shaken_status plan_step_launch(Plan& P, cudaStream_t st, uint64_t* nl,
   uint64_t count = 0;
   const bool timed = P.timing > 0 && !capturing && P.steps_issued % (uint64_t)P.timing == 0;
   if (!capturing) ++P.steps_issued;
-  bool obs_needed = false, track = false;
+  bool lattice_sums = false, graph_sums = false, track = false;
   int ex = 0;
   for (shaken_ctx* c : P.members) {
     // multispin lattices track with the observables kernel; graphs fuse tracking
     // into half 0 unless a per-step series (which also needs M) is recorded
     if (c->hcd.tracking && c->kind == SHAKEN_LATTICE && c->enc == SHAKEN_MULTISPIN)
-      obs_needed = true;
-    if (c->hcd.tracking && c->kind == SHAKEN_GRAPH && c->hcd.record) obs_needed = true;
+      lattice_sums = true;
+    if (c->kind == SHAKEN_GRAPH && P.cl_clusters > 0) continue;  // tracked in its own run
+    if (c->hcd.tracking && c->kind == SHAKEN_GRAPH && c->hcd.record) graph_sums = true;
     if (c->hcd.tracking && c->kind == SHAKEN_GRAPH && !c->hcd.record) track = true;
     ex |= c->exact_always;
   }
-  if (obs_needed) {
-    for (auto& F : P.fams) {
-      if (F->kind == 0 && F->enc == SHAKEN_MULTISPIN) {
-        CU(shk::launch_lattice_obs(F->enc, F->wpt, F->jobs.as<LatJob>(), F->tiles.as<Tile>(),
-                                   F->n_tiles, 0, 0, st));
-        ++count;
-      } else if (F->kind == 1) {
-        TRY(graph_obs(*F, 0, 0, st, &count));
-      }
+  for (auto& F : P.fams) {
+    if (F->kind == 0 && F->enc == SHAKEN_MULTISPIN && lattice_sums) {
+      CU(shk::launch_lattice_obs(F->enc, F->wpt, F->jobs.as<LatJob>(), F->tiles.as<Tile>(),
+                                 F->n_tiles, 0, 0, st));
+      ++count;
+    } else if (F->kind == 1 && graph_sums) {
+      TRY(graph_obs(*F, 0, 0, st, &count));
     }
   }
   for (uint32_t half = 0; half < 2; ++half) {
@@ -834,6 +888,15 @@ static shaken_status plan_run(Plan& P, cudaStream_t st, uint64_t n_steps, bool u
                               uint64_t* nl) {
   if (P.dirty) TRY(build_plan(P, st));
   uint64_t done = 0;
+  if (P.cl_clusters > 0) {
+    for (uint64_t k = 0; k < n_steps; k += 1u << 16) {
+      CU(shk::launch_graph_cluster(P.cl_jobs.as<GraphJob>(), P.cl_clusters, P.cl_n, P.cl_m,
+                                   P.cl_blocks, P.cl_ctx.as<CtxDev*>(), P.cl_n_ctx,
+                                   (uint32_t)std::min<uint64_t>(n_steps - k, 1u << 16), st));
+      *nl += 2;
+    }
+    if (P.n_ctx == 0) return SHAKEN_OK;  // no other members
+  }
   if (use_graph && n_steps >= (uint64_t)kGraphChunk) {
     if (!P.gexec) {
       cudaStream_t cap = nullptr;
@@ -2068,6 +2131,7 @@ shaken_status shaken_batch_set_timing(shaken_batch* b, int on) {
   CU(cudaStreamSynchronize(b->stream));
   b->plan.collect();
   if (on < 0) return fail(SHAKEN_E_INVAL, "timing stride must be >= 0");
+  if ((b->plan.timing > 0) != (on > 0)) b->plan.invalidate();  // timed plans run half step by half step
   b->plan.timing = on;
   b->plan.steps_issued = 0;
   b->plan.timed_ms = 0.0;
