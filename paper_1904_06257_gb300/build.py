@@ -16,7 +16,8 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libshaken.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
-SOURCES = ["lattice.cu", "lattice_cluster.cu", "graph.cu", "graph_sliced.cu", "graph_cluster.cu", "graph_obs.cu", "misc.cu", "noalloc.cu", "runtime.cu"]
+SOURCES = ["lattice.cu", "lattice_cluster.cu", "lattice_ahead.cu",
+           "graph.cu", "graph_sliced.cu", "graph_cluster.cu", "graph_obs.cu", "misc.cu", "noalloc.cu", "runtime.cu"]
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 
 

@@ -67,6 +67,12 @@ int lattice_cluster_shape(uint32_t, int, double*);
 cudaError_t launch_lattice_cluster(const LatJob*, int, uint32_t, int, uint32_t, uint32_t, cudaStream_t);
 cudaError_t launch_lattice_resident(int, const LatJob*, int, uint32_t, uint32_t, uint32_t,
                                     cudaStream_t);
+uint32_t lattice_ahead_chunk(int, int, uint32_t, uint64_t, size_t*);
+bool lattice_ahead_faster(int, int, uint32_t);
+cudaError_t launch_lattice_ahead(int, const LatJob*, int, uint32_t, uint32_t, uint32_t, void*,
+                                 cudaStream_t);
+cudaError_t launch_lattice_follow(int, int, const LatJob*, int, uint32_t, uint32_t, uint32_t,
+                                  const void*, cudaStream_t);
 cudaError_t launch_philox(uint64_t, const uint32_t*, uint32_t*, int64_t, cudaStream_t);
 cudaError_t launch_threshold(const double*, const double*, uint64_t*, int64_t, cudaStream_t);
 }  // namespace shk
@@ -273,6 +279,7 @@ struct shaken_ctx {
                                                    // threshold classes
   std::vector<uint32_t> hubs[2];  // graph: (x, first edge, end edge) of the vertices of degree
                                   // above kHubDeg, in-CSR [0] and out-CSR [1]
+  DevMem ahead;                // outcome words of a chunk of steps (small lattices' whole runs)
   DevMem band_xch, band_sync;  // banded runs: row exchange area and grid barrier
   int cluster = -1;            // MULTISPIN whole runs: blocks per cluster (0: no; -1: not known yet)
   double cluster_us = 0.0;     // and the time of a step that way
@@ -1371,6 +1378,9 @@ static bool resident_eligible(const shaken_ctx* c, uint64_t n_steps) {
   return (uint64_t)c->L * c->L / 32 <= 4096;
 }
 
+// Field classes of different thresholds: by n + s where q = J, else by (n, s).
+static int field_classes(const shaken_ctx* c) { return c->q == c->J ? 4 : 6; }
+
 // Small MULTISPIN lattices: one thread-block cluster per group of 32 replicas, where that takes
 // less time per step than the kernels of a step on the whole GPU.  Both in microseconds per
 // step, fitted to sides 32 .. 256 and 1 .. 64 groups: a half step in a cluster is its chain
@@ -1390,28 +1400,57 @@ static bool cluster_eligible(shaken_ctx* c, uint64_t n_steps) {
   return c->cluster_us + (tr ? 1.0 : 0.0) < (tr ? 18.5 : 8.5) + (tr ? 3.6e-5 : 2.2e-5) * words;
 }
 
+// Steps of a chunk of a run with the draws compared ahead of it (lattice_ahead.cu), whose outcome
+// words c->ahead then holds; 0: not that way (too many words, or no memory for them).
+static uint32_t ahead_chunk(shaken_ctx* c, int nc, int n_jobs, uint32_t words, uint64_t n_steps) {
+  size_t bytes = 0;
+  const uint32_t chunk = shk::lattice_ahead_chunk(nc, n_jobs, words, n_steps, &bytes);
+  if (chunk == 0 || (c->ahead.bytes < bytes && c->ahead.alloc(bytes) != SHAKEN_OK)) return 0;
+  return chunk;
+}
+
 static shaken_status run_resident(shaken_ctx* c, uint64_t n_steps) {
   cudaStream_t st = c->stream;
   if (c->solo.dirty) TRY(build_plan(c->solo, st));
   const Family& F = *c->solo.fams[0];
-  const bool cluster = c->enc == SHAKEN_MULTISPIN;
-  const int n_jobs = cluster ? c->R / 32 : c->R;
   const uint32_t words = (uint32_t)(c->L * c->L / 32);
+  const int nc = field_classes(c);
+  uint32_t ahead = 0;
+  if (shk::lattice_ahead_faster(nc, c->R, words))
+    ahead = ahead_chunk(c, nc, c->R, words, n_steps);
   uint64_t done = 0;
   while (done < n_steps) {
-    const uint64_t chunk = std::min<uint64_t>(n_steps - done, 1u << 16);
+    const uint32_t chunk =
+        (uint32_t)std::min<uint64_t>(n_steps - done, ahead > 0 ? ahead : 1u << 16);
     const uint32_t t = (uint32_t)(c->host_step + done);
-    if (cluster)
-      CU(shk::launch_lattice_cluster(F.jobs.as<LatJob>(), n_jobs, (uint32_t)c->L, c->cluster, t,
-                                     (uint32_t)chunk, st));
-    else
-      CU(shk::launch_lattice_resident(F.enc, F.jobs.as<LatJob>(), n_jobs, words, t,
-                                      (uint32_t)chunk, st));
-    c->launches++;
+    if (ahead > 0) {
+      CU(shk::launch_lattice_ahead(nc, F.jobs.as<LatJob>(), c->R, words, t, chunk, c->ahead.p, st));
+      CU(shk::launch_lattice_follow(F.enc, nc, F.jobs.as<LatJob>(), c->R, words, t, chunk,
+                                    c->ahead.p, st));
+    } else {
+      CU(shk::launch_lattice_resident(F.enc, F.jobs.as<LatJob>(), c->R, words, t, chunk, st));
+    }
+    c->launches += ahead > 0 ? 2 : 1;
     done += chunk;
   }
   c->host_step += n_steps;
   return push_cd(c);  // the device step counter follows the host's
+}
+
+static shaken_status run_cluster(shaken_ctx* c, uint64_t n_steps) {
+  cudaStream_t st = c->stream;
+  if (c->solo.dirty) TRY(build_plan(c->solo, st));
+  const Family& F = *c->solo.fams[0];
+  uint64_t done = 0;
+  while (done < n_steps) {
+    const uint64_t chunk = std::min<uint64_t>(n_steps - done, 1u << 16);
+    CU(shk::launch_lattice_cluster(F.jobs.as<LatJob>(), c->R / 32, (uint32_t)c->L, c->cluster,
+                                   (uint32_t)(c->host_step + done), (uint32_t)chunk, st));
+    c->launches++;
+    done += chunk;
+  }
+  c->host_step += n_steps;
+  return push_cd(c);
 }
 
 // Mid-size single lattices (INT8/PACKED, one replica, beyond the resident size)
@@ -1466,8 +1505,8 @@ static shaken_status run_band(shaken_ctx* c, uint64_t n_steps, int grid, size_t 
 }
 
 static shaken_status solo_run(shaken_ctx* ctx, uint64_t n_steps) {
-  if (resident_eligible(ctx, n_steps) || cluster_eligible(ctx, n_steps))
-    return run_resident(ctx, n_steps);
+  if (resident_eligible(ctx, n_steps)) return run_resident(ctx, n_steps);
+  if (cluster_eligible(ctx, n_steps)) return run_cluster(ctx, n_steps);
   int grid = 0;
   size_t smem = 0;
   if (band_eligible(ctx, n_steps, &grid, &smem)) return run_band(ctx, n_steps, grid, smem);
