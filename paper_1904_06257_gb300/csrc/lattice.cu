@@ -1074,7 +1074,30 @@ __global__ void __launch_bounds__(kTile, kBandMinBlocks) lattice_band_kernel(
   (void)calls;
 }
 
+// --------------------------------------------------------------------------- bit copies
+// The INT8 state as bit lane words (lane word w: bytes 32 w .. 32 w + 31) and back: bound by HBM.
+__global__ void __launch_bounds__(kTile) to_bits_kernel(const uint4* __restrict__ bytes,
+                                                        uint32_t* __restrict__ words, size_t n) {
+  const size_t w = (size_t)blockIdx.x * kTile + threadIdx.x;
+  if (w < n) words[w] = bits32(__ldcs(bytes + 2 * w), __ldcs(bytes + 2 * w + 1));
+}
+
+__global__ void __launch_bounds__(kTile) to_bytes_kernel(const uint32_t* __restrict__ words,
+                                                         uint4* __restrict__ bytes, size_t n) {
+  const size_t k = (size_t)blockIdx.x * kTile + threadIdx.x;  // half a word each: whole lines
+  if (k < 2 * n) __stcs(bytes + k, bytes16(__ldg(words + (k >> 1)) >> (16u * (k & 1u))));
+}
+
 // --------------------------------------------------------------------------- launchers
+cudaError_t launch_bits(int pack, const uint4* from, uint32_t* words, uint4* to, size_t n,
+                        cudaStream_t st) {
+  if (pack)
+    to_bits_kernel<<<(unsigned)((n + kTile - 1) / kTile), kTile, 0, st>>>(from, words, n);
+  else
+    to_bytes_kernel<<<(unsigned)((2 * n + kTile - 1) / kTile), kTile, 0, st>>>(words, to, n);
+  return cudaGetLastError();
+}
+
 static int grid_for(int n_tiles, int per_sm) {
   int dev = 0, sms = 152;
   cudaGetDevice(&dev);

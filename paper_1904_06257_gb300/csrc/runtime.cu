@@ -73,6 +73,7 @@ cudaError_t launch_lattice_ahead(int, const LatJob*, int, uint32_t, uint32_t, ui
                                  cudaStream_t);
 cudaError_t launch_lattice_follow(int, int, const LatJob*, int, uint32_t, uint32_t, uint32_t,
                                   const void*, cudaStream_t);
+cudaError_t launch_bits(int, const uint4*, uint32_t*, uint4*, size_t, cudaStream_t);
 cudaError_t launch_philox(uint64_t, const uint32_t*, uint32_t*, int64_t, cudaStream_t);
 cudaError_t launch_threshold(const double*, const double*, uint64_t*, int64_t, cudaStream_t);
 }  // namespace shk
@@ -177,6 +178,7 @@ struct Family {
 struct Plan {
   std::vector<shaken_ctx*> members;
   std::vector<std::unique_ptr<Family>> fams;
+  std::vector<std::unique_ptr<Family>> bits;  // INT8 lattice: its half steps on the bit copy
   DevMem ctxlist;
   int n_ctx = 0;
   // graph members stepped in whole runs, one cluster of cl_blocks blocks per group (cl_clusters
@@ -279,6 +281,7 @@ struct shaken_ctx {
                                                    // threshold classes
   std::vector<uint32_t> hubs[2];  // graph: (x, first edge, end edge) of the vertices of degree
                                   // above kHubDeg, in-CSR [0] and out-CSR [1]
+  DevMem bits;                 // INT8: sigma and sigma' as bit lane words, during a run on them
   DevMem ahead;                // outcome words of a chunk of steps (small lattices' whole runs)
   DevMem band_xch, band_sync;  // banded runs: row exchange area and grid barrier
   int cluster = -1;            // MULTISPIN whole runs: blocks per cluster (0: no; -1: not known yet)
@@ -598,13 +601,13 @@ static void choose_clusters(Plan& P) {
 
 static shaken_status build_plan(Plan& P, cudaStream_t st) {
   P.fams.clear();
+  P.bits.clear();
   P.drop_graph();
   choose_clusters(P);
   std::vector<std::vector<LatJob>> ljobs(3);
   std::vector<std::vector<GraphJob>> gjobs(2);  // 0 integer, 1 real: half-step jobs
   std::vector<std::vector<GraphJob>> ojobs(2);  // per-group jobs
   std::vector<std::vector<Tile>> otiles(2);
-  std::vector<std::vector<Tile>> tiles(3);
   std::vector<Tile> gtiles[2][2], vtiles[2], stiles[2][2][shk::kSlicedShapes];  // [family][half], [.][.][shape]
   std::vector<std::vector<HubItem>> hitems(2);    // per graph family: hub chunks
   std::vector<std::vector<uint32_t>> hunits(2);   // unit -> item
@@ -733,23 +736,33 @@ static shaken_status build_plan(Plan& P, cudaStream_t st) {
       }
     }
   }
-  LatShape lat_shape[3];
-  for (int e = 0; e < 3; ++e) {
-    if (ljobs[e].empty()) continue;
-    TRY(choose_lattice_shape(P, e, ljobs[e], st, &lat_shape[e]));
-    lattice_tiles(ljobs[e], (uint32_t)(kTile * lat_shape[e].wpt), tiles[e]);
-  }
-  for (int e = 0; e < 3; ++e) {
-    if (ljobs[e].empty()) continue;
+  auto lattice_family = [&](int e, const std::vector<LatJob>& jobs,
+                            std::vector<std::unique_ptr<Family>>& fams) -> shaken_status {
+    LatShape shape;
+    std::vector<Tile> tiles;
+    TRY(choose_lattice_shape(P, e, jobs, st, &shape));
+    lattice_tiles(jobs, (uint32_t)(kTile * shape.wpt), tiles);
     auto F = std::make_unique<Family>();
     F->kind = 0;
     F->enc = e;
-    F->wpt = lat_shape[e].wpt;
-    F->bps = lat_shape[e].bps;
-    TRY(upload(F->jobs, ljobs[e].data(), ljobs[e].size() * sizeof(LatJob), st));
-    TRY(upload(F->tiles, tiles[e].data(), tiles[e].size() * sizeof(Tile), st));
-    F->n_tiles = (int)tiles[e].size();
-    P.fams.push_back(std::move(F));
+    F->wpt = shape.wpt;
+    F->bps = shape.bps;
+    TRY(upload(F->jobs, jobs.data(), jobs.size() * sizeof(LatJob), st));
+    TRY(upload(F->tiles, tiles.data(), tiles.size() * sizeof(Tile), st));
+    F->n_tiles = (int)tiles.size();
+    fams.push_back(std::move(F));
+    return SHAKEN_OK;
+  };
+  for (int e = 0; e < 3; ++e)
+    if (!ljobs[e].empty()) TRY(lattice_family(e, ljobs[e], P.fams));
+  if (P.members.size() == 1 && &P == &P.members[0]->solo && P.members[0]->bits.p != nullptr) {
+    std::vector<LatJob> jobs(ljobs[SHAKEN_INT8]);  // the same jobs on the bit copy
+    uint32_t* w = P.members[0]->bits.as<uint32_t>();
+    for (size_t j = 0; j < jobs.size(); ++j) {
+      jobs[j].A = w + j * jobs[j].nwords;
+      jobs[j].B = w + (jobs.size() + j) * jobs[j].nwords;
+    }
+    TRY(lattice_family(SHAKEN_PACKED, jobs, P.bits));
   }
   for (int fi = 0; fi < 2; ++fi) {
     if (gjobs[fi].empty()) continue;
@@ -1504,6 +1517,34 @@ static shaken_status run_band(shaken_ctx* c, uint64_t n_steps, int grid, size_t 
   return push_cd(c);  // the device step counter follows the host's
 }
 
+// INT8 runs of the half-step kernels go through the PACKED ones on a bit copy of the state: the draws
+// of the two encodings are the same, and a byte word costs twice a bit word (conversions to bits
+// and back on three loads and a store).  The copies cost the bytes once (16 ns per 1000 lane words,
+// three launches); a step saves 30: at L = 16384 470 -> 215 us.  Fewer steps, and timed or counted
+// runs, stay on the bytes.
+static bool bits_eligible(const shaken_ctx* c, uint64_t n_steps) {
+  if (c->kind != SHAKEN_LATTICE || c->owner || c->enc != SHAKEN_INT8 || n_steps < 2) return false;
+  if (c->solo.timing > 0 || c->solo.rng_counter != nullptr) return false;
+  const double words = (double)c->spin_bytes / 32.0;
+  return (double)n_steps * 3.0e-5 * words > 8.0 + 1.6e-5 * words;
+}
+
+static shaken_status run_bits(shaken_ctx* c, uint64_t n_steps, uint64_t* nl) {
+  cudaStream_t st = c->stream;
+  if (c->solo.dirty) TRY(build_plan(c->solo, st));
+  const size_t words = c->spin_bytes / 32;
+  uint32_t* w = c->bits.as<uint32_t>();
+  CU(shk::launch_bits(1, c->A.as<uint4>(), w, nullptr, words, st));
+  std::swap(c->solo.fams, c->solo.bits);
+  const shaken_status s = plan_run(c->solo, st, n_steps, n_steps >= 64, nl);
+  std::swap(c->solo.fams, c->solo.bits);
+  if (s != SHAKEN_OK) return s;
+  CU(shk::launch_bits(0, nullptr, w, c->A.as<uint4>(), words, st));
+  CU(shk::launch_bits(0, nullptr, w + words, c->B.as<uint4>(), words, st));
+  *nl += 3;
+  return SHAKEN_OK;
+}
+
 static shaken_status solo_run(shaken_ctx* ctx, uint64_t n_steps) {
   if (resident_eligible(ctx, n_steps)) return run_resident(ctx, n_steps);
   if (cluster_eligible(ctx, n_steps)) return run_cluster(ctx, n_steps);
@@ -1511,7 +1552,13 @@ static shaken_status solo_run(shaken_ctx* ctx, uint64_t n_steps) {
   size_t smem = 0;
   if (band_eligible(ctx, n_steps, &grid, &smem)) return run_band(ctx, n_steps, grid, smem);
   uint64_t nl = 0;
-  shaken_status s = plan_run(ctx->solo, ctx->stream, n_steps, n_steps >= 64, &nl);
+  bool bits = bits_eligible(ctx, n_steps);
+  if (bits && ctx->bits.p == nullptr) {  // no memory for the copy: on the bytes
+    bits = ctx->bits.alloc(ctx->spin_bytes / 4) == SHAKEN_OK;
+    if (bits) ctx->solo.invalidate();
+  }
+  const shaken_status s = bits ? run_bits(ctx, n_steps, &nl)
+                               : plan_run(ctx->solo, ctx->stream, n_steps, n_steps >= 64, &nl);
   ctx->launches += nl;
   if (s != SHAKEN_OK) return s;
   ctx->host_step += n_steps;
