@@ -139,6 +139,7 @@ struct DevMem {
     bytes = n;
     return SHAKEN_OK;
   }
+  shaken_status reserve(size_t n) { return p != nullptr && bytes >= n ? SHAKEN_OK : alloc(n); }
   template <class T>
   T* as() const {
     return static_cast<T*>(p);
@@ -173,6 +174,16 @@ struct Family {
   // (chunk, group) unit; partial rows and finished-chunk counters of their words
   DevMem hub_items, hub_units, hub_partial, hub_done;
   int n_hub_units = 0;
+  void reset() {  // all but the device buffers
+    wpt = 1;
+    bps = n_tiles = n_otiles = n_hub_units = 0;
+    for (int h = 0; h < 2; ++h) {
+      for (Range& r : stiles[h]) r = Range{};
+      gtiles[h] = Range{};
+    }
+    vtiles = Range{};
+    fields = false;
+  }
 };
 
 struct Plan {
@@ -600,8 +611,23 @@ static void choose_clusters(Plan& P) {
 }
 
 static shaken_status build_plan(Plan& P, cudaStream_t st) {
+  // the families of the last build keep their device buffers (a plan is rebuilt at the beginning
+  // and the end of every anneal and recorded run: 30 us of allocations each time otherwise)
+  std::vector<std::unique_ptr<Family>> old(std::move(P.fams));
+  for (auto& f : P.bits) old.push_back(std::move(f));
   P.fams.clear();
   P.bits.clear();
+  auto family = [&](int kind, int enc) {
+    for (auto& f : old)
+      if (f && f->kind == kind && f->enc == enc) {
+        f->reset();
+        return std::move(f);
+      }
+    auto f = std::make_unique<Family>();
+    f->kind = kind;
+    f->enc = enc;
+    return f;
+  };
   P.drop_graph();
   choose_clusters(P);
   std::vector<std::vector<LatJob>> ljobs(3);
@@ -742,9 +768,7 @@ static shaken_status build_plan(Plan& P, cudaStream_t st) {
     std::vector<Tile> tiles;
     TRY(choose_lattice_shape(P, e, jobs, st, &shape));
     lattice_tiles(jobs, (uint32_t)(kTile * shape.wpt), tiles);
-    auto F = std::make_unique<Family>();
-    F->kind = 0;
-    F->enc = e;
+    auto F = family(0, e);
     F->wpt = shape.wpt;
     F->bps = shape.bps;
     TRY(upload(F->jobs, jobs.data(), jobs.size() * sizeof(LatJob), st));
@@ -766,9 +790,7 @@ static shaken_status build_plan(Plan& P, cudaStream_t st) {
   }
   for (int fi = 0; fi < 2; ++fi) {
     if (gjobs[fi].empty()) continue;
-    auto F = std::make_unique<Family>();
-    F->kind = 1;
-    F->enc = fi == 0 ? 1 : 0;
+    auto F = family(1, fi == 0 ? 1 : 0);
     TRY(upload(F->jobs, gjobs[fi].data(), gjobs[fi].size() * sizeof(GraphJob), st));
     std::vector<Tile> all;
     auto put = [&](const std::vector<Tile>& t) {
@@ -797,8 +819,8 @@ static shaken_status build_plan(Plan& P, cudaStream_t st) {
     if (!hunits[fi].empty()) {
       TRY(upload(F->hub_items, hitems[fi].data(), hitems[fi].size() * sizeof(HubItem), st));
       TRY(upload(F->hub_units, hunits[fi].data(), hunits[fi].size() * 4, st));
-      TRY(F->hub_partial.alloc((size_t)hrows[fi] * 32u * 4u));
-      TRY(F->hub_done.alloc((size_t)hdone[fi] * 4u));
+      TRY(F->hub_partial.reserve((size_t)hrows[fi] * 32u * 4u));
+      TRY(F->hub_done.reserve((size_t)hdone[fi] * 4u));
       CU(cudaMemsetAsync(F->hub_done.p, 0, (size_t)hdone[fi] * 4u, st));
       F->n_hub_units = (int)hunits[fi].size();
     }
@@ -1633,14 +1655,16 @@ shaken_status shaken_anneal(shaken_ctx* ctx, const double* beta_schedule, uint64
   return end_anneal(ctx);
 }
 
+static constexpr size_t kSeriesKept = 8u << 20;  // bytes of a series buffer kept for the next run
+
 shaken_status shaken_step_record(shaken_ctx* ctx, uint64_t n_steps, double* mag, double* energy) {
   if (!ctx) return fail(SHAKEN_E_INVAL, "ctx is NULL");
   if (ctx->owner) return fail(SHAKEN_E_STATE, "context belongs to a batch");
   TRY(check_steps(ctx, n_steps));
   if (n_steps == 0) return SHAKEN_OK;
   const size_t bytes = (size_t)n_steps * ctx->R * sizeof(double);
-  TRY(ctx->series_m.alloc(bytes));
-  TRY(ctx->series_H.alloc(bytes));
+  TRY(ctx->series_m.reserve(bytes));
+  TRY(ctx->series_H.reserve(bytes));
   ctx->hcd.record = 1u;
   ctx->hcd.series_t0 = (uint32_t)ctx->host_step;
   ctx->hcd.series_cap = (uint32_t)n_steps;
@@ -1660,8 +1684,8 @@ shaken_status shaken_step_record(shaken_ctx* ctx, uint64_t n_steps, double* mag,
   ctx->hcd.tracking = ctx->tracking ? 1u : 0u;
   ctx->solo.invalidate();
   TRY(push_cd(ctx));
-  ctx->series_m.release();
-  ctx->series_H.release();
+  if (ctx->series_m.bytes > kSeriesKept) ctx->series_m.release();
+  if (ctx->series_H.bytes > kSeriesKept) ctx->series_H.release();
   return SHAKEN_OK;
 }
 
