@@ -1,25 +1,31 @@
 // graph_cluster.cu -- whole runs of small +-1 graphs: one thread-block cluster owns one group of
-// 32 replicas of a graph for n steps, its words in the blocks' shared memory.
+// 32 replicas of a graph for a chunk of steps, its words in the blocks' shared memory, the draws
+// compared ahead of the run.
 //
-// Vertex x's word lives in block x mod C (C a power of two), so neighbours are gathered
-// from distributed shared memory; 32 consecutive slots of the degree order make a warp's
-// pass, dealt round the blocks.  A block keeps its slots' entries and columns of both
-// directions in shared memory, too (lane-major per pass): read from global memory they
-// came from L2 in every half step, since the cluster barrier empties L1.  The first pass's
-// two Philox calls of the next half step are made between arriving at the barrier and
-// waiting for it.  A half step ends at the cluster barrier.  Draws, classes and
-// decisions are those of graph_sliced_kernel, so the trajectory is the same.  One lambda on
-// all vertices: the class bytes of the next step (by degree) are made during the second
-// half step.  With tracking the agreeing edges of sigma_t are counted in the first
+// A draw depends on (seed, vertex, group, step, half) alone and a threshold on the class (agreeing
+// neighbours, own spin) alone, so the outcome of every class is known before the configuration is.
+// graph_thresholds_kernel makes the thresholds of a chunk of steps (fp64, by degree and class),
+// graph_ahead_kernel the outcome words of every vertex and class on the whole GPU, and
+// graph_cluster_kernel only counts neighbours and selects.  The outcomes are those of all 32
+// planes, so the trajectory is that of the half-step kernels.
+//
+// Every block holds all of the group's words, so neighbours are gathers from its own shared
+// memory.  32 consecutive slots of a direction's degree order make a warp's pass, dealt
+// round the blocks; the buffer a half step writes is in the order of its own direction, so a
+// pass's results are one line to each block (distributed shared memory).  A block keeps
+// the entries and columns of its slots in both directions in shared memory, too, as places in
+// the buffer that the half step reads (lane-major per pass).  The outcome words of a
+// warp's next pass are on their way (cp.async) during a pass.  A half step ends at the
+// cluster barrier.  With tracking the agreeing edges of sigma_t are counted in the first
 // half, gathered by the cluster's first block during the second and turned into best
 // energies and series behind the next barrier (lambda = 0).
 //
-// Bound by a half step's chain: barrier, entry and column loads, gathers, two Philox calls,
-// the plane comparison, a round of queued lanes -- about 1250 instructions of the warps that have
-// vertices, one of them at a time on a scheduler (7 cycles each).  n = 2000, mean degree 6,
-// 32 replicas, tracked anneal: 11 us a step in clusters of 16 (14 us in clusters of 4),
-// against 19 us of the half-step kernels and 37 us of the general kernel.
+// Bound by a half step's chain (barrier, gathers, selects, stores to the other blocks).  n = 2000,
+// mean degree 6, 32 replicas, 200 annealed steps: 4.5 us a step; 6.3 with each word in one block,
+// gathered from distributed shared memory (5 ns a vertex of a block against 1.4); 10.6 with the draws
+// made in the run; 19 in the half-step kernels.  n = 8000: 7.0 against 20.6 us.
 #include <cooperative_groups.h>
+#include <cuda_pipeline_primitives.h>
 
 #include <cstdint>
 
@@ -30,67 +36,145 @@ namespace shk {
 
 namespace cg = cooperative_groups;
 
-constexpr int kGclThreads = 256;  // 255 registers a thread: local memory is as far as L2 here
+constexpr int kGclThreads = 512;
 constexpr int kGclWarps = kGclThreads / 32;
+constexpr int kAheadThreads = 256;  // of graph_ahead_kernel
 constexpr int kGclPlanes = 10;  // counter planes: at most kGclPasses passes of degree <= 31
 constexpr int kGclPasses = 32;
 constexpr uint32_t kGclColSlack = 3 * 32 * 31;  // see gcl_col_words
+constexpr int kGclDegs = 32, kGclClasses = 32;  // degrees 0..31, classes of a vertex at most
 
 struct GclShared {
-  __align__(16) uint8_t by_deg[2][32][32];  // [step parity][degree][class] top bytes, bit-reversed
   GraphJob J;
-  uint32_t amb[2][32];       // classes of uncertain top byte, by degree
-  uint2 q[kGclWarps][64];
-  uint2 key[10];
-  double beta[2];            // by step parity
-  float kb[2];
   uint32_t base[2][kGclPasses * kGclWarps];  // first padded column word of a pass, per direction
+  uint8_t ncls[2][kGclPasses * kGclWarps];   // most classes of a pass's vertices
   unsigned int block[2][32];  // up spins and agreeing edges of this block's vertices, per replica
   unsigned int all[2][32];    // of the cluster (used in block 0)
 };
+
+// Classes of a vertex of degree d: i = a + [sigma = +1] at q = 1 (a agreeing in-neighbours;
+// the field of (a, +1) is that of (a + 1, -1) exactly), else 2 a + [sigma = +1].
+__device__ __forceinline__ uint32_t gcl_classes(bool collapse, uint32_t d) {
+  return collapse ? d + 2u : 2u * d + 2u;
+}
+
+// T of every degree and class for step cd->step + k of a context (the block of its first group):
+// tab[((job n_steps + k) 32 + d) 32 + i] = (low word, ~0 where T = 2^32); without an anneal
+// all steps share step 0's.
+__global__ void __launch_bounds__(128) graph_thresholds_kernel(const GraphJob* __restrict__ jobs,
+                                                               uint32_t n_steps,
+                                                               uint2* __restrict__ tab) {
+  const uint32_t job = blockIdx.x / n_steps, k = blockIdx.x % n_steps;
+  const GraphJob& J = jobs[job];
+  if (J.g0 != 0u) return;
+  const CtxDev* cd = J.cd;
+  const uint32_t t = cd->step + k, anneal_len = cd->anneal_len;
+  const bool anneal = J.beta_sched != nullptr && anneal_len != 0u;
+  if (t >= cd->t_end || (k != 0u && !anneal)) return;
+  const double beta =
+      anneal ? J.beta_sched[min(t - cd->anneal_t0, anneal_len - 1u)] : J.beta_lane[0];
+  const uint32_t dmax = max(J.in_visit[J.n - 1u].z, J.out_visit[J.n - 1u].z);
+  const bool collapse = J.q == 1.0;
+  uint2* out = tab + (size_t)blockIdx.x * (kGclDegs * kGclClasses);
+  for (uint32_t o = threadIdx.x; o < (dmax + 1u) * kGclClasses; o += blockDim.x) {
+    const uint32_t d = o / kGclClasses, i = o % kGclClasses;
+    if (d >= (uint32_t)kGclDegs || i >= gcl_classes(collapse, d)) continue;
+    const int a = (int)(collapse ? i : i >> 1), up = collapse ? 0 : (int)(i & 1u);
+    const double h = field_h(1.0, 2 * a - (int)d, J.q, 2 * up - 1, (double)J.lambda_c);
+    const unsigned long long T = threshold_T(h, beta);
+    out[o] = make_uint2((uint32_t)T, T >> 32 != 0ull ? 0xffffffffu : 0u);
+  }
+}
+
+// Outcomes u < T of every class, one warp per pass of 32 slots of a half step's degree order:
+// out[((k 2 + pos) ptot + off[job] + pass) stride + 32 i + lane] for class i.
+// Bound by integer issue: three Philox calls and, a class, four operations a plane.
+// (8000 vertices, 4 groups, mean degree 8: 180 ns per 1000 words and step.)
+__global__ void __launch_bounds__(kAheadThreads) graph_ahead_kernel(
+    const GraphJob* __restrict__ jobs, const uint32_t* __restrict__ off, uint32_t n_steps,
+    uint32_t per, uint32_t ptot, uint32_t stride, const uint2* __restrict__ tab,
+    uint32_t* __restrict__ out) {
+  uint32_t item = blockIdx.x / per;
+  const uint32_t pass = (blockIdx.x % per) * (kAheadThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31u;
+  const uint32_t pos = item & 1u, k = (item >> 1) % n_steps, job = (item >> 1) / n_steps;
+  const GraphJob& J = jobs[job];
+  const CtxDev* cd = J.cd;
+  const uint32_t t = cd->step + k, n = J.n, s = pass * 32u + lane;
+  if (t >= cd->t_end || pass * 32u >= n) return;
+  const uint32_t typ = pos ^ cd->order;
+  const bool anneal = J.beta_sched != nullptr && cd->anneal_len != 0u;
+  const bool in = s < n;
+  const uint4 vi = in ? (typ == 0u ? J.in_visit : J.out_visit)[s] : make_uint4(0u, 0u, 0u, 0u);
+  const uint32_t x = vi.x, ncls = in ? gcl_classes(J.q == 1.0, vi.z) : 0u;
+  const uint32_t F = in && J.frozen != nullptr ? __ldg(J.frozen + x) : 0u;
+  const PhKey K = ph_key(J.key0, J.key1);
+  const PhShared P = ph_shared(K, J.g0, t);
+  const uint4 W[3] = {ph_call_shared(K, P, x, typ), ph_call_shared(K, P, x, typ + 2u),
+                      ph_call_shared(K, P, x, typ + 4u)};
+  const uint2* T = tab + ((size_t)(job - J.g0) * n_steps + (anneal ? k : 0u)) *
+                             (kGclDegs * kGclClasses) + vi.z * kGclClasses;
+  uint32_t* o = out + ((size_t)(2u * k + pos) * ptot + off[job] + pass) * stride + lane;
+  const uint32_t most = __reduce_max_sync(0xffffffffu, ncls);
+#pragma unroll 1
+  for (uint32_t i = 0; i < most; ++i) {
+    const uint2 th = i < ncls ? __ldg(T + i) : make_uint2(0u, 0xffffffffu);
+    uint32_t lt = 0u, eq = 0xffffffffu;
+#pragma unroll
+    for (int j = 11; j >= 0; --j) {  // twelve planes as a subtraction: borrow and equality
+      const uint4& q = W[j >> 2];
+      const uint32_t w = (j & 3) == 0 ? q.x : (j & 3) == 1 ? q.y : (j & 3) == 2 ? q.z : q.w;
+      const uint32_t m = (uint32_t)((int32_t)(th.x << j) >> 31);
+      lt = maj3(~w, m, lt);
+      eq &= ~(w ^ m);
+    }
+    const uint32_t sure = F | th.y;
+    lt &= ~eq;
+    eq &= ~sure;
+#pragma unroll 1
+    for (uint32_t call = 3; call < 8u && eq != 0u; ++call) {
+      const uint4 q = ph_call_shared(K, P, x, typ + 2u * call);
+#pragma unroll
+      for (uint32_t b = 0; b < 4u; ++b) {
+        const uint32_t w = b == 0u ? q.x : b == 1u ? q.y : b == 2u ? q.z : q.w;
+        const uint32_t m = (uint32_t)((int32_t)(th.x << (4u * call + b)) >> 31);
+        const uint32_t diff = (w ^ m) & eq;
+        lt |= diff & m;
+        eq &= ~diff;
+      }
+    }
+    if (i < ncls) o[32u * i] = lt | sure;
+  }
+}
+
+// Class idx (planes I) of the 2^NB outcome words p[32 i].
+template <int NB>
+__device__ __forceinline__ uint32_t gcl_select(const uint32_t* p, const uint32_t (&I)[kIdx]) {
+  if constexpr (NB == 0) {
+    return *p;
+  } else {
+    const uint32_t lo = gcl_select<NB - 1>(p, I), hi = gcl_select<NB - 1>(p + (32 << (NB - 1)), I);
+    return (I[NB - 1] & hi) | (~I[NB - 1] & lo);
+  }
+}
 
 __device__ __forceinline__ uint32_t dsm_addr(uint32_t local, uint32_t rank) {
   uint32_t a;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(local), "r"(rank));
   return a;
 }
-__device__ __forceinline__ uint32_t dsm_ld(uint32_t a) {
-  uint32_t v;
-  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
-  return v;
-}
 __device__ __forceinline__ void dsm_st(uint32_t a, uint32_t v) {
   asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-}
-__device__ __forceinline__ void dsm_or(uint32_t a, uint32_t v) {
-  asm volatile("red.relaxed.cluster.shared::cluster.or.b32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
 __device__ __forceinline__ void dsm_add(uint32_t a, uint32_t v) {
   asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
 
-// Up to 32 queued lanes (entries as in graph_sliced_kernel, without the group).
-__device__ __noinline__ void gcl_round(const GclShared& sh, const uint4* entry, const uint2* q,
-                                       int cnt, uint32_t dst, uint32_t t, uint32_t typ,
-                                       uint32_t C, uint32_t lc, int lane) {
-  __syncwarp();
-  if (lane < cnt) {
-    const uint2 e = q[lane];
-    const GraphJob& J = sh.J;
-    const uint4 vi = entry[e.x];
-    const int k = (int)(e.y & 31u);
-    if (sliced_lane(J.key0, J.key1, vi.x, J.g0, t, typ, J.q, J.q == 1.0, sh.kb[t & 1u],
-                    sh.beta[t & 1u], (int)vi.z, __uint_as_float(vi.w), k, (e.y >> 5) & 31u,
-                    (e.y >> 18) & 0xFFu, ((e.y >> 26) & 1u) != 0u))
-      dsm_or(dsm_addr(dst + 4u * (vi.x >> lc), vi.x & (C - 1u)), 1u << k);
-  }
-  __syncwarp();
-}
-
 // jobs: one per group (g0); n_steps: at most, a context stops at its t_end; col_words: the
-// padded column words of a direction that the shared memory holds.
+// padded column words of a direction that the shared memory holds; off, ptot, stride, ahead: the
+// outcome words (graph_ahead_kernel).
 __global__ void __launch_bounds__(kGclThreads, 1) graph_cluster_kernel(
-    const GraphJob* __restrict__ jobs, uint32_t n_steps, uint32_t col_words) {
+    const GraphJob* __restrict__ jobs, const uint32_t* __restrict__ off, uint32_t n_steps,
+    uint32_t col_words, uint32_t ptot, uint32_t stride, const uint32_t* __restrict__ ahead) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   GclShared& sh = *reinterpret_cast<GclShared*>(smem_raw);
   uint32_t* words = reinterpret_cast<uint32_t*>(smem_raw + (sizeof(GclShared) + 15) / 16 * 16);
@@ -107,30 +191,31 @@ __global__ void __launch_bounds__(kGclThreads, 1) graph_cluster_kernel(
   const uint32_t t0 = cd->step, t_end = cd->t_end, order = cd->order;
   if (t0 >= t_end) return;  // every block of the cluster
   const uint32_t steps = min(n_steps, t_end - t0);
-  const uint32_t n = J.n, nper = (n + C - 1u) >> lc, g = J.g0, G = J.G;
-  const uint32_t anneal_t0 = cd->anneal_t0, anneal_len = cd->anneal_len;
-  const bool anneal = J.beta_sched != nullptr && anneal_len != 0u;
+  const uint32_t n = J.n, g = J.g0, G = J.G;
   const bool track = cd->tracking && J.sums != nullptr, record = track && cd->record;
-  const bool collapse = J.q == 1.0, qint = J.q == rint(J.q);
-  const uint32_t buf0 = (uint32_t)__cvta_generic_to_shared(words);
-  if (tid < 10)
-    sh.key[tid] = make_uint2(J.key0 + (uint32_t)tid * kPhW0, J.key1 + (uint32_t)tid * kPhW1);
-  for (uint32_t i = (uint32_t)tid; i < nper; i += kGclThreads) {
-    const uint32_t x = (i << lc) + r;
-    words[i] = x < n ? J.A[(size_t)x * G + g] : 0u;
-  }
-  // beta, and the class bytes by degree (eight threads a degree), of step t
-  // the block's slots of both directions: entries (vertex, -, degree, lambda), columns
+  const bool collapse = J.q == 1.0;
+  const uint32_t* const mine = ahead + (size_t)off[blockIdx.x / C] * stride;
   const uint32_t chunks = (n + 31u) / 32u;                    // passes of the whole graph
   const uint32_t mine_n = chunks > r ? (chunks - r + C - 1u) >> lc : 0u;  // of this block: j = i C + r
-  const uint32_t slots = ((chunks + C - 1u) >> lc) * 32u;
-  uint4* const entries = reinterpret_cast<uint4*>(words + ((2u * nper + 3u) & ~3u));
-  uint32_t* const columns = reinterpret_cast<uint32_t*>(entries + 2u * slots);
+  const uint32_t slots = ((chunks + C - 1u) >> lc) * 32u, nw = 32u * chunks;
+  uint32_t* const entries = words + 2u * nw;
+  uint32_t* const stages = entries + 2u * slots;  // two a warp
+  uint32_t* const columns = stages + 2u * kGclWarps * stride + 32u * kGclClasses;
+  const uint32_t words_at = (uint32_t)__cvta_generic_to_shared(words);
+  auto visits = [&](uint32_t dir) { return dir == 0u ? J.in_visit : J.out_visit; };
+  // each vertex's slot in both orders, where the words will be
+  for (uint32_t dir = 0; dir < 2u; ++dir)
+    for (uint32_t s = (uint32_t)tid; s < n; s += kGclThreads)
+      words[dir * nw + visits(dir)[s].x] = s;
+  __syncthreads();
+  // the block's slots of both directions: entries (own word in the buffer read | degree << 24),
+  // columns (neighbour's word | sign of J)
   for (uint32_t dir = 0; dir < 2u; ++dir) {
-    const uint4* visit = dir == 0u ? J.in_visit : J.out_visit;
+    const uint32_t* at = words + (dir ^ 1u) * nw;
     for (uint32_t o = (uint32_t)tid; o < mine_n * 32u; o += kGclThreads) {
       const uint32_t s = ((o >> 5) * C + r) * 32u + (o & 31u);
-      entries[dir * slots + o] = s < n ? visit[s] : make_uint4(0u, 0u, 0u, 0u);
+      const uint4 vi = s < n ? visits(dir)[s] : make_uint4(0u, 0u, 0u, 0u);
+      entries[dir * slots + o] = at[vi.x] | vi.z << 24;
     }
   }
   __syncthreads();
@@ -141,7 +226,9 @@ __global__ void __launch_bounds__(kGclThreads, 1) graph_cluster_kernel(
       uint32_t v = 0u;
       if (i < mine_n) {
         const uint32_t last = min(31u, n - 1u - (i * C + r) * 32u);
-        v = 32u * entries[(uint32_t)warp * slots + i * 32u + last].z;
+        const uint32_t d = entries[(uint32_t)warp * slots + i * 32u + last] >> 24;
+        v = 32u * d;
+        sh.ncls[warp][i] = (uint8_t)gcl_classes(collapse, d);
       }
       uint32_t sum = v;
 #pragma unroll
@@ -155,37 +242,23 @@ __global__ void __launch_bounds__(kGclThreads, 1) graph_cluster_kernel(
   }
   __syncthreads();
   for (uint32_t dir = 0; dir < 2u; ++dir) {
+    const uint32_t* at = words + (dir ^ 1u) * nw;
     const uint32_t* col = dir == 0u ? J.in_col : J.out_col;
     for (uint32_t o = (uint32_t)tid; o < mine_n * 32u; o += kGclThreads) {
-      const uint4 vi = entries[dir * slots + o];
+      const uint32_t s = ((o >> 5) * C + r) * 32u + (o & 31u);
+      if (s >= n) continue;
+      const uint4 vi = visits(dir)[s];
       uint32_t* c = columns + dir * col_words + sh.base[dir][o >> 5] + (o & 31u);
-      for (uint32_t e = 0; e < vi.z; ++e) c[32u * e] = __ldg(col + vi.y + e);
+      for (uint32_t e = 0; e < vi.z; ++e) {
+        const uint32_t v = __ldg(col + vi.y + e);
+        c[32u * e] = at[v & 0x7fffffffu] | (v & 0x80000000u);
+      }
     }
   }
-  auto beta_of = [&](uint32_t t) {
-    uint32_t k = t - anneal_t0;
-    if (k >= anneal_len) k = anneal_len - 1u;
-    return anneal ? __ldg(J.beta_sched + k) : __ldg(J.beta_lane + 32u * g);
-  };
-  auto stage = [&](uint32_t t, double b) {
-    const float kb = (float)(-2.0 * b * 1.4426950408889634);
-    if (tid == 0) {
-      sh.beta[t & 1u] = b;
-      sh.kb[t & 1u] = kb;
-    }
-    {
-      const uint32_t d = (uint32_t)tid >> 3, ncls = collapse ? d + 2u : 2u * d + 2u;
-      uint32_t mine = 0u;
-      for (uint32_t i = (uint32_t)tid & 7u; i < min(ncls, 32u); i += 8u)
-        mine |= sliced_class(J.q, collapse, qint, kb, i, d, J.lambda_c, sh.by_deg[t & 1u][d]) << i;
-#pragma unroll
-      for (int s = 1; s < 8; s <<= 1) mine |= __shfl_xor_sync(0xffffffffu, mine, s);
-      if ((tid & 7) == 0) sh.amb[t & 1u][d] = mine;
-    }
-  };
-  double b_next = beta_of(t0 + 1u);  // read a step ahead
-  stage(t0, beta_of(t0));
-  if (!anneal) stage(t0 + 1u, b_next);
+  __syncthreads();
+  // buffer 0 (sigma) is written by the step's second half, buffer 1 (sigma') by its first
+  for (uint32_t s = (uint32_t)tid; s < n; s += kGclThreads)
+    words[s] = J.A[(size_t)visits(order ^ 1u)[s].x * G + g];
   const bool keeper = track && r == 0u && tid >= kGclThreads - 32;
   const uint32_t fwd = (uint32_t)tid - (kGclThreads - 96u);  // < 64: forwards the block's sums
   const uint32_t rep = 32u * g + (uint32_t)lane;
@@ -213,33 +286,29 @@ __global__ void __launch_bounds__(kGclThreads, 1) graph_cluster_kernel(
     }
   };
   cl.sync();
-  SlicedWord<1> w;
-  uint2* q = sh.q[warp];
-  const uint32_t below = (1u << lane) - 1u;
-  // the parts of a step's Philox calls that all vertices share
-  auto philox_step = [&](uint32_t t) {
-    const unsigned long long p1 = (unsigned long long)kPhM1 * t;
-    w.u1 = (uint32_t)p1;
-    const unsigned long long pm = (unsigned long long)kPhM0 * ((uint32_t)(p1 >> 32) ^ g ^ J.key0);
-    w.h01[0] = (uint32_t)(pm >> 32);
-    w.l01[0] = (uint32_t)pm;
+  // the outcome words of pass i of a half step into one of the warp's stages
+  uint32_t* const stage = stages + 2u * (uint32_t)warp * stride;
+  uint32_t flip = 0u;
+  auto fetch = [&](uint32_t st, uint32_t pos, uint32_t i) {
+    if (i < mine_n && st < steps) {
+      const uint32_t* src = mine + ((size_t)(2u * st + pos) * ptot + i * C + r) * stride;
+      uint32_t* dst = stage + flip * stride;
+      const uint32_t chunks16 = 8u * sh.ncls[pos ^ order][i];
+      for (uint32_t c = (uint32_t)lane; c < chunks16; c += 32u)
+        __pipeline_memcpy_async(dst + 4u * c, src + 4u * c, 16);
+    }
+    __pipeline_commit();
+    flip ^= 1u;
   };
-  uint32_t ahead[2][4][1];  // the first pass's calls
-  auto call_ahead = [&](uint32_t typ) {
-    if ((uint32_t)warp >= mine_n) return;
-    w.x = entries[typ * slots + (uint32_t)tid].x;
-    sliced_call<1>(sh.key, w, typ, ahead[0]);
-    sliced_call<1>(sh.key, w, typ + 2u, ahead[1]);
-  };
-  philox_step(t0);
-  call_ahead(order);
+  if ((uint32_t)warp < mine_n) fetch(0u, 0u, (uint32_t)warp);
 #pragma unroll 1
   for (uint32_t st = 0; st < steps; ++st) {
     const uint32_t t = t0 + st;
 #pragma unroll 1
     for (uint32_t pos = 0; pos < 2u; ++pos) {
       const uint32_t typ = pos ^ order;
-      const uint32_t src = buf0 + 4u * nper * pos, dst = buf0 + 4u * nper * (pos ^ 1u);
+      const uint32_t* src = words + nw * pos;
+      const uint32_t dst = words_at + 4u * nw * (pos ^ 1u);
       const bool sums = track && pos == 0u;
       if (keeper && pos == 0u && st != 0u) close(t - 1u);
       if (track && pos == 1u && fwd < 64u) {  // this block's sums to block 0
@@ -249,44 +318,42 @@ __global__ void __launch_bounds__(kGclThreads, 1) graph_cluster_kernel(
         if (v != 0u)
           dsm_add(dsm_addr((uint32_t)__cvta_generic_to_shared(&sh.all[0][0] + fwd), 0u), v);
       }
-      int qn = 0;
       uint32_t cnt[kGclPlanes], bound = 0u, ups[6] = {0u, 0u, 0u, 0u, 0u, 0u};
 #pragma unroll
       for (int b = 0; b < kGclPlanes; ++b) cnt[b] = 0u;
 #pragma unroll 1
       for (uint32_t i = (uint32_t)warp; i < mine_n; i += (uint32_t)kGclWarps) {
         const uint32_t local = 32u * i + (uint32_t)lane;
+        const bool more = i + (uint32_t)kGclWarps < mine_n;
+        fetch(more || pos == 0u ? st : st + 1u, more ? pos : pos ^ 1u,
+              more ? i + (uint32_t)kGclWarps : (uint32_t)warp);
         const bool in = (i * C + r) * 32u + (uint32_t)lane < n;
-        const uint4 vi = entries[typ * slots + local];
+        const uint32_t entry = entries[typ * slots + local];
         const uint32_t* col = columns + typ * col_words + sh.base[typ][i] + lane;
-        w.x = vi.x;
-        const uint32_t d = vi.z;
-        const uint32_t S = in ? dsm_ld(dsm_addr(src + 4u * (w.x >> lc), w.x & (C - 1u))) : 0u;
-        uint32_t I[kIdx][1];
+        const uint32_t d = entry >> 24;
+        const uint32_t S = in ? src[entry & 0xffffffu] : 0u;
+        uint32_t I[kIdx];
 #pragma unroll
-        for (int b = 0; b < kIdx; ++b) I[b][0] = 0u;
+        for (int b = 0; b < kIdx; ++b) I[b] = 0u;
 #pragma unroll 1
         for (uint32_t e = 0; e < d; e += 4) {  // four edges at a time, the last again beyond d
           uint32_t cv[4], x[4];
 #pragma unroll
           for (uint32_t k = 0; k < 4; ++k) cv[k] = col[32u * min(e + k, d - 1u)];
 #pragma unroll
-          for (uint32_t k = 0; k < 4; ++k) {
-            const uint32_t y = cv[k] & 0x7fffffffu;
-            x[k] = dsm_ld(dsm_addr(src + 4u * (y >> lc), y & (C - 1u)));
-          }
+          for (uint32_t k = 0; k < 4; ++k) x[k] = src[cv[k] & 0x7fffffffu];
 #pragma unroll
           for (uint32_t k = 0; k < 4; ++k)
             x[k] = e + k < d ? x[k] ^ (uint32_t)((int32_t)cv[k] >> 31) : 0u;
-          const uint32_t s0 = I[0][0] ^ x[0] ^ x[1], ca = maj3(I[0][0], x[0], x[1]);
+          const uint32_t s0 = I[0] ^ x[0] ^ x[1], ca = maj3(I[0], x[0], x[1]);
           const uint32_t cb = maj3(s0, x[2], x[3]);
-          I[0][0] = s0 ^ x[2] ^ x[3];
-          uint32_t c = maj3(I[1][0], ca, cb);
-          I[1][0] ^= ca ^ cb;
+          I[0] = s0 ^ x[2] ^ x[3];
+          uint32_t c = maj3(I[1], ca, cb);
+          I[1] ^= ca ^ cb;
 #pragma unroll
           for (int b = 2; b < kIdx; ++b) {
-            const uint32_t u = I[b][0] & c;
-            I[b][0] ^= c;
+            const uint32_t u = I[b] & c;
+            I[b] ^= c;
             c = u;
           }
         }
@@ -296,7 +363,7 @@ __global__ void __launch_bounds__(kGclThreads, 1) graph_cluster_kernel(
           for (int b = 0; b < kGclPlanes; ++b) {
             uint32_t ag = 0u;
             if (b < kIdx) {
-              const uint32_t D = 0u - ((d >> b) & 1u), A = I[b][0];
+              const uint32_t D = 0u - ((d >> b) & 1u), A = I[b];
               ag = (S & A) | (~S & (D ^ A ^ br));
               br = (~D & A) | (~D & br) | (A & br);
             }
@@ -313,80 +380,34 @@ __global__ void __launch_bounds__(kGclThreads, 1) graph_cluster_kernel(
             c = u;
           }
         }
-        uint32_t ncls = 0u;
         if (collapse) {  // idx = a + sigma
           uint32_t c = S;
 #pragma unroll
           for (int b = 0; b < kIdx; ++b) {
-            const uint32_t u = I[b][0] & c;
-            I[b][0] ^= c;
+            const uint32_t u = I[b] & c;
+            I[b] ^= c;
             c = u;
           }
-          ncls = d + 2u;
         } else {  // idx = 2 a + sigma
 #pragma unroll
-          for (int b = kIdx - 1; b > 0; --b) I[b][0] = I[b - 1][0];
-          I[0][0] = S;
-          ncls = 2u * d + 2u;
+          for (int b = kIdx - 1; b > 0; --b) I[b] = I[b - 1];
+          I[0] = S;
         }
-        const uint8_t* tbv = sh.by_deg[t & 1u][d];
-        w.vamb = sh.amb[t & 1u][d];
-        w.F = in ? (J.frozen != nullptr ? __ldg(J.frozen + w.x) : 0u) : 0xffffffffu;
-        const uint32_t nm = __reduce_max_sync(0xffffffffu, ncls);
-        uint32_t lt[1] = {0u}, eq[1] = {~w.F};
-#pragma unroll 1
-        for (int call = 1; call >= 0; --call) {
-          uint32_t o[4][1];
-          if (i < (uint32_t)kGclWarps) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) o[k][0] = call != 0 ? ahead[1][k][0] : ahead[0][k][0];
-          } else {
-            sliced_call<1>(sh.key, w, typ + 2u * (uint32_t)call, o);
-          }
-          if (nm <= 4u)
-            sliced_planes<2, 1>(tbv, call, I, o, lt, eq);
-          else if (nm <= 8u)
-            sliced_planes<3, 1>(tbv, call, I, o, lt, eq);
-          else if (nm <= 16u)
-            sliced_planes<4, 1>(tbv, call, I, o, lt, eq);
-          else
-            sliced_planes<5, 1>(tbv, call, I, o, lt, eq);
+        __pipeline_wait_prior(1);
+        __syncwarp();
+        const uint32_t* o = stage + flip * stride + lane;  // the stage before the one in flight
+        const uint32_t nm = sh.ncls[typ][i];
+        const uint32_t res = nm <= 4u    ? gcl_select<2>(o, I)
+                             : nm <= 8u  ? gcl_select<3>(o, I)
+                             : nm <= 16u ? gcl_select<4>(o, I)
+                                         : gcl_select<5>(o, I);
+        if (in) {  // to every block
+          const uint32_t to = dst + 4u * ((i * C + r) * 32u + (uint32_t)lane);
+#pragma unroll 4
+          for (uint32_t c = 0; c < C; ++c) dsm_st(dsm_addr(to, (r + c) & (C - 1u)), res);
         }
-        uint32_t amb = 0u;
-#pragma unroll 1
-        for (uint32_t m = w.vamb; m != 0u; m &= m - 1u) {  // rare: lanes of uncertain classes
-          const uint32_t c = (uint32_t)__ffs(m) - 1u;
-          uint32_t is = 0xffffffffu;
-#pragma unroll
-          for (int b = 0; b < kIdx; ++b) is &= ~(I[b][0] ^ (0u - ((c >> b) & 1u)));
-          amb |= is;
-        }
-        uint32_t und = (eq[0] | amb) & ~w.F;
-        if (in)
-          dsm_st(dsm_addr(dst + 4u * (w.x >> lc), w.x & (C - 1u)), (lt[0] & ~und) | w.F);
-#pragma unroll 1
-        while (true) {  // one undecided lane of each thread at a time
-          const uint32_t ball = __ballot_sync(0xffffffffu, und != 0u);
-          if (ball == 0u) break;
-          if (und != 0u) {
-            const int k = __ffs(und) - 1;
-            und &= und - 1u;
-            uint32_t idx = 0u;
-#pragma unroll
-            for (int b = 0; b < kIdx; ++b) idx |= ((I[b][0] >> k) & 1u) << b;
-            q[qn + __popc(ball & below)] =
-                make_uint2(local, (uint32_t)k | (idx << 5) |
-                                     ((__brev((uint32_t)tbv[idx]) >> 24) << 18) |
-                                     (((w.vamb >> idx) & 1u) << 26));
-          }
-          qn += __popc(ball);
-          if (qn >= 32) {
-            qn -= 32;
-            gcl_round(sh, entries + typ * slots, q + qn, 32, dst, t, typ, C, lc, lane);
-          }
-        }
+        __syncwarp();  // before the stage is filled again
       }
-      if (qn > 0) gcl_round(sh, entries + typ * slots, q, qn, dst, t, typ, C, lc, lane);
       if (sums && bound != 0u) {  // the warp's threads: per-replica counts of its planes
         uint32_t cm = 0u, ce = 0u;
 #pragma unroll
@@ -399,23 +420,15 @@ __global__ void __launch_bounds__(kGclThreads, 1) graph_cluster_kernel(
         }
         if (ce) atomicAdd(&sh.block[1][lane], ce);
       }
-      if (anneal && pos == 1u) {  // the next step's thresholds
-        stage(t + 1u, b_next);
-        b_next = beta_of(t + 2u);
-      }
-      cl.barrier_arrive();
-      if (pos == 1u) philox_step(t + 1u);
-      call_ahead(typ ^ 1u);  // the next half step's (the next step begins with the other type)
-      cl.barrier_wait();
+      cl.sync();
     }
   }
   if (keeper) close(t0 + steps - 1u);
-  for (uint32_t i = (uint32_t)tid; i < nper; i += kGclThreads) {
-    const uint32_t x = (i << lc) + r;
-    if (x < n) {
-      J.A[(size_t)x * G + g] = words[i];
-      J.B[(size_t)x * G + g] = words[nper + i];
-    }
+  for (uint32_t o = (uint32_t)tid; o < mine_n * 32u; o += kGclThreads) {
+    const uint32_t s = ((o >> 5) * C + r) * 32u + (o & 31u);
+    if (s >= n) continue;
+    J.A[(size_t)visits(order ^ 1u)[s].x * G + g] = words[s];
+    J.B[(size_t)visits(order)[s].x * G + g] = words[nw + s];
   }
 }
 
@@ -435,20 +448,24 @@ static uint32_t gcl_col_words(uint64_t m, uint32_t C) {
   return (uint32_t)(m / C) + kGclColSlack;
 }
 
-static size_t gcl_bytes(uint32_t n, uint64_t m, uint32_t C) {
-  const size_t nper = (n + C - 1u) / C, slots = ((n + 31u) / 32u + C - 1u) / C * 32u;
-  return (sizeof(GclShared) + 15) / 16 * 16 + (2 * nper + 3) / 4 * 16 + 2 * slots * sizeof(uint4) +
+// Words of a pass's outcomes.
+static uint32_t gcl_stride(int classes) { return 32u * (uint32_t)classes; }
+
+static size_t gcl_bytes(uint32_t n, uint64_t m, uint32_t C, int classes) {
+  const size_t chunks = (n + 31u) / 32u, slots = (chunks + C - 1u) / C * 32u;
+  return (sizeof(GclShared) + 15) / 16 * 16 + 2 * 32 * chunks * sizeof(uint32_t) + 2 * slots * sizeof(uint32_t) +
+         (2 * kGclWarps * gcl_stride(classes) + 32 * kGclClasses) * sizeof(uint32_t) +
          2 * (size_t)gcl_col_words(m, C) * sizeof(uint32_t);
 }
 
 static cudaError_t gcl_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, uint32_t n,
-                              uint64_t m, uint32_t C, int clusters, cudaStream_t st) {
-  const size_t bytes = gcl_bytes(n, m, C);
-  cudaError_t e = cudaFuncSetAttribute(graph_cluster_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+                              uint64_t m, uint32_t C, int classes, int clusters, cudaStream_t st) {
+  const size_t bytes = gcl_bytes(n, m, C, classes);
+  const auto kernel = graph_cluster_kernel;
+  cudaError_t e =
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(graph_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed,
-                             1);
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
   cfg = cudaLaunchConfig_t{};
   cfg.gridDim = dim3((unsigned)clusters * C);
@@ -464,26 +481,29 @@ static cudaError_t gcl_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr
 }
 
 // Blocks per cluster for `clusters` groups of graphs of at most n vertices, and the microseconds
-// of a step: the size of least time, a half step taking 2.5 us and 11.5 ns per vertex of a
-// block, times the waves of clusters (as in lattice_cluster_shape); 0: too large.
-int graph_cluster_shape(uint32_t n, uint64_t m, int clusters, double* us) {
+// of a step: the size of least time, a half step taking 0.8 us, 1.45 ns per vertex of a block
+// and, in clusters, 0.1 ns per vertex of the graph (results stored to every block), times the
+// waves of clusters (as in lattice_cluster_shape); 0: too large.  Fitted to 100 steps of n = 500 ..
+// 10000; one group of n = 2000 with 1, 2, 4, 8, 16 blocks: 7.8, 5.3, 3.8, 3.5, 3.7 us a step.
+int graph_cluster_shape(uint32_t n, uint64_t m, int classes, int clusters, double* us) {
   int dev = 0, max_smem = 0, best = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   for (uint32_t C = 1; C <= 16u; C *= 2) {
     const uint32_t passes = (n + C * kGclThreads - 1u) / (C * kGclThreads);
-    if (gcl_bytes(n, m, C) + 1024 > (size_t)max_smem || passes > (uint32_t)kGclPasses) continue;
+    if (gcl_bytes(n, m, C, classes) + 1024 > (size_t)max_smem || passes > (uint32_t)kGclPasses) continue;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
     int fit = 0;
-    if (gcl_config(cfg, attr, n, m, C, clusters, nullptr) != cudaSuccess ||
+    if (gcl_config(cfg, attr, n, m, C, classes, clusters, nullptr) != cudaSuccess ||
         cudaOccupancyMaxActiveClusters(&fit, graph_cluster_kernel, &cfg) != cudaSuccess ||
         fit < 1) {
       cudaGetLastError();
       continue;
     }
     const int wave = C == 1u || fit < 4 ? fit : fit * 3 / 4;
-    const double t = 2.0 * (2.5 + 1.15e-2 * n / C) * ((clusters + wave - 1) / wave);
+    const double t = 2.0 * (0.8 + 1.45e-3 * n / C + (C > 1u ? 1e-4 * n : 0.0)) *
+                     ((clusters + wave - 1) / wave);
     if (best == 0 || t < *us) {
       best = (int)C;
       *us = t;
@@ -492,13 +512,31 @@ int graph_cluster_shape(uint32_t n, uint64_t m, int clusters, double* us) {
   return best;
 }
 
-cudaError_t launch_graph_cluster(const GraphJob* jobs, int clusters, uint32_t n, uint64_t m, int C,
-                                 CtxDev* const* ctxs, int n_ctx, uint32_t steps, cudaStream_t st) {
+// Bytes of the outcome words and thresholds of a step.
+size_t graph_cluster_step_bytes(int classes, int clusters, uint32_t ptot) {
+  return (size_t)2 * ptot * gcl_stride(classes) * sizeof(uint32_t) +
+         (size_t)clusters * kGclDegs * kGclClasses * sizeof(uint2);
+}
+
+// `steps` steps (the work buffer holds that many: graph_cluster_step_bytes each) of `clusters`
+// groups; off: first pass of each group among ptot.
+cudaError_t launch_graph_cluster(const GraphJob* jobs, const uint32_t* off, int clusters, uint32_t n,
+                                 uint64_t m, int classes, uint32_t ptot, int C, CtxDev* const* ctxs,
+                                 int n_ctx, uint32_t steps, void* work, cudaStream_t st) {
   if (clusters <= 0 || steps == 0) return cudaSuccess;
+  const uint32_t stride = gcl_stride(classes);
+  uint32_t* const out = static_cast<uint32_t*>(work);
+  uint2* const tab = reinterpret_cast<uint2*>(out + (size_t)2 * steps * ptot * stride);
+  graph_thresholds_kernel<<<(unsigned)clusters * steps, 128, 0, st>>>(jobs, steps, tab);
+  const uint32_t per = ((n + 31u) / 32u + kAheadThreads / 32 - 1u) / (kAheadThreads / 32);
+  graph_ahead_kernel<<<(unsigned)clusters * steps * 2u * per, kAheadThreads, 0, st>>>(
+      jobs, off, steps, per, ptot, stride, tab, out);
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
-  cudaError_t e = gcl_config(cfg, attr, n, m, (uint32_t)C, clusters, st);
-  if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, graph_cluster_kernel, jobs, steps, gcl_col_words(m, (uint32_t)C));
+  cudaError_t e = gcl_config(cfg, attr, n, m, (uint32_t)C, classes, clusters, st);
+  if (e == cudaSuccess)
+    e = cudaLaunchKernelEx(&cfg, graph_cluster_kernel, jobs, off, steps,
+                           gcl_col_words(m, (uint32_t)C), ptot, stride, (const uint32_t*)out);
   if (e != cudaSuccess) return e;
   advance_kernel<<<(n_ctx + 127) / 128, 128, 0, st>>>(ctxs, n_ctx, steps);
   return cudaGetLastError();

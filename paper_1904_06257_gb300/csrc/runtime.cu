@@ -45,9 +45,10 @@ cudaError_t launch_graph_half(bool, const GraphJob*, const Tile*, int, uint32_t,
 cudaError_t launch_graph_sliced(int, bool, const GraphJob*, const Tile*, int, uint32_t,
                                 cudaStream_t);
 int graph_sliced_blocks(int, bool);
-int graph_cluster_shape(uint32_t, uint64_t, int, double*);
-cudaError_t launch_graph_cluster(const GraphJob*, int, uint32_t, uint64_t, int, CtxDev* const*, int,
-                                 uint32_t, cudaStream_t);
+int graph_cluster_shape(uint32_t, uint64_t, int, int, double*);
+size_t graph_cluster_step_bytes(int, int, uint32_t);
+cudaError_t launch_graph_cluster(const GraphJob*, const uint32_t*, int, uint32_t, uint64_t, int,
+                                 uint32_t, int, CtxDev* const*, int, uint32_t, void*, cudaStream_t);
 int graph_half_blocks();
 cudaError_t launch_graph_hub(bool, const GraphJob*, const HubItem*, const uint32_t*, int, uint32_t,
                              uint32_t*, uint32_t*, cudaStream_t);
@@ -194,10 +195,13 @@ struct Plan {
   int n_ctx = 0;
   // graph members stepped in whole runs, one cluster of cl_blocks blocks per group (cl_clusters
   // of them, cl_n_ctx members of at most cl_n vertices and cl_m edges); the others: ctxlist
-  DevMem cl_jobs, cl_ctx;
-  int cl_clusters = 0, cl_blocks = 0, cl_n_ctx = 0;
-  uint32_t cl_n = 0;
+  // vertices have at most cl_classes classes; cl_off: a group's first 32-vertex pass among
+  // cl_passes; cl_work: the outcome words of up to cl_chunk steps
+  DevMem cl_jobs, cl_ctx, cl_off, cl_work;
+  int cl_clusters = 0, cl_blocks = 0, cl_n_ctx = 0, cl_classes = 0;
+  uint32_t cl_n = 0, cl_passes = 0, cl_chunk = 0;
   uint64_t cl_m = 0;
+  bool cl_refused = false;  // no memory for cl_work
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
   int graph_steps = 0;
@@ -290,6 +294,7 @@ struct shaken_ctx {
   uint32_t sliced_slots[2][2] = {{0, 0}, {0, 0}};  // graph: slots of the degree order (in, out)
                                                    // whose vertices have at most 16, 32
                                                    // threshold classes
+  int32_t max_deg = 0;            // graph: largest in- or out-degree
   std::vector<uint32_t> hubs[2];  // graph: (x, first edge, end edge) of the vertices of degree
                                   // above kHubDeg, in-CSR [0] and out-CSR [1]
   DevMem bits;                 // INT8: sigma and sigma' as bit lane words, during a run on them
@@ -572,21 +577,26 @@ static shaken_status choose_lattice_shape(const Plan& P, int enc, const std::vec
 
 // Whether the graph members of a plan are stepped in whole runs by graph_cluster_kernel: +-1
 // couplings, one lambda, every vertex and half step within the bit-sliced kernel, and less
-// time per step than the half-step kernels and the epilogue, which take 18 us (a small job's three
-// chains of launches and dependent loads) and 50 ns per 1000 words.  Measured on both sides of the
-// line, 100 tracked steps of mean degree 8: n = 4000, one group 1790 (cluster) against 2470 us,
-// eight groups 1890 against 2680; n = 16000, one group 3330 against 2540.  (With a lambda per
-// vertex the class bytes of a thread's vertex are its own work: 2350 against 1810 us at
-// n = 4000.)  Sets the plan's cluster size.
+// time per step than the half-step kernels and the epilogue.  The run takes its chain
+// (shk::graph_cluster_shape), the outcome words made ahead (29 ns per 1000 words and class) and a
+// chunk's launches and loads; the half-step kernels 14.3 us and 40 ns per 1000 words, tracked
+// 18 us and 60 ns.  Measured on both sides of the line, mean degree 8, 200 annealed steps:
+// n = 8000, four groups 11.2 (cluster) against 21.2 us a step, eight groups 19.5 against 24.1;
+// 100 plain steps: 10.3 against 16.3, eight groups 17.9 against 17.6.  (With a lambda per vertex
+// the thresholds would be each vertex's own.)  Sets the plan's cluster size.
+static constexpr size_t kClusterWork = 64u << 20;  // bytes of outcome words, at most (stay in L2)
+
 static void choose_clusters(Plan& P) {
   P.cl_clusters = P.cl_blocks = P.cl_n_ctx = 0;
   P.cl_n = 0;
   P.cl_m = 0;
+  if (P.cl_refused) return;
   if (P.timing > 0) return;  // timed runs bracket the half-step launches
-  double words = 0.0;
-  int clusters = 0, members = 0;
+  double words = 0.0, outcomes = 0.0;
+  bool tracked = false;
+  int clusters = 0, members = 0, classes = 2;
   uint32_t most = 0;
-  uint64_t edges = 0;
+  uint64_t edges = 0, passes = 0;
   for (const shaken_ctx* c : P.members) {
     if (c->kind != SHAKEN_GRAPH) continue;
     if (c->n > (int64_t)1 << 20 || !sliced_half(c, 0) || !sliced_half(c, 1) ||
@@ -596,13 +606,25 @@ static void choose_clusters(Plan& P) {
     ++members;
     clusters += c->R / 32;
     words += (double)c->n * (c->R / 32);
+    passes += (uint64_t)((c->n + 31) / 32) * (c->R / 32);
+    outcomes += ((c->q == 1.0 ? 1.0 : 2.0) * (double)c->m + 2.0 * (double)c->n) * (c->R / 32);
+    tracked = tracked || c->hcd.tracking;
+    classes = std::max(classes, c->q == 1.0 ? c->max_deg + 2 : 2 * c->max_deg + 2);
     most = std::max(most, (uint32_t)c->n);
     edges = std::max(edges, (uint64_t)c->m);
   }
   if (members == 0 || clusters > 1024) return;
   double us = 0.0;
-  const int blocks = shk::graph_cluster_shape(most, edges, clusters, &us);
-  if (blocks == 0 || us >= 18.0 + 5e-5 * words) return;
+  if (passes > 1u << 20 || classes > 32) return;
+  const int blocks = shk::graph_cluster_shape(most, edges, classes, clusters, &us);
+  const size_t step = shk::graph_cluster_step_bytes(classes, clusters, (uint32_t)passes);
+  const uint32_t chunk = (uint32_t)std::min<size_t>(kClusterWork / step, 64);
+  if (blocks == 0 || chunk == 0) return;
+  us += 2.9e-5 * outcomes + (8.0 + 6e-4 * most) / chunk;
+  if (us >= (tracked ? 18.0 + 6e-5 * words : 14.3 + 4e-5 * words)) return;
+  P.cl_classes = classes;
+  P.cl_passes = (uint32_t)passes;
+  P.cl_chunk = chunk;
   P.cl_clusters = clusters;
   P.cl_blocks = blocks;
   P.cl_n_ctx = members;
@@ -831,6 +853,13 @@ static shaken_status build_plan(Plan& P, cudaStream_t st) {
   if (P.cl_clusters > 0) {
     TRY(upload(P.cl_jobs, ojobs[0].data(), ojobs[0].size() * sizeof(GraphJob), st));
     TRY(upload(P.cl_ctx, cl_cds.data(), cl_cds.size() * sizeof(CtxDev*), st));
+    std::vector<uint32_t> off;
+    uint32_t first = 0;
+    for (const GraphJob& J : ojobs[0]) {
+      off.push_back(first);
+      first += (J.n + 31u) / 32u;
+    }
+    TRY(upload(P.cl_off, off.data(), off.size() * sizeof(uint32_t), st));
   }
   P.dirty = false;
   return SHAKEN_OK;
@@ -931,11 +960,25 @@ static shaken_status plan_run(Plan& P, cudaStream_t st, uint64_t n_steps, bool u
   if (P.dirty) TRY(build_plan(P, st));
   uint64_t done = 0;
   if (P.cl_clusters > 0) {
-    for (uint64_t k = 0; k < n_steps; k += 1u << 16) {
-      CU(shk::launch_graph_cluster(P.cl_jobs.as<GraphJob>(), P.cl_clusters, P.cl_n, P.cl_m,
-                                   P.cl_blocks, P.cl_ctx.as<CtxDev*>(), P.cl_n_ctx,
-                                   (uint32_t)std::min<uint64_t>(n_steps - k, 1u << 16), st));
-      *nl += 2;
+    const size_t work =
+        shk::graph_cluster_step_bytes(P.cl_classes, P.cl_clusters, P.cl_passes) *
+        (size_t)std::min<uint64_t>(n_steps, P.cl_chunk);
+    // with room for a batch that grows by members
+    size_t room = 1u << 20;
+    while (room < work) room *= 2;
+    if (P.cl_work.bytes < work && P.cl_work.alloc(room) != SHAKEN_OK) {
+      P.cl_refused = true;  // the half-step kernels take no such buffer
+      TRY(build_plan(P, st));
+    }
+  }
+  if (P.cl_clusters > 0) {
+    for (uint64_t k = 0; k < n_steps; k += P.cl_chunk) {
+      CU(shk::launch_graph_cluster(P.cl_jobs.as<GraphJob>(), P.cl_off.as<uint32_t>(), P.cl_clusters,
+                                   P.cl_n, P.cl_m, P.cl_classes, P.cl_passes, P.cl_blocks,
+                                   P.cl_ctx.as<CtxDev*>(), P.cl_n_ctx,
+                                   (uint32_t)std::min<uint64_t>(n_steps - k, P.cl_chunk),
+                                   P.cl_work.p, st));
+      *nl += 4;
     }
     if (P.n_ctx == 0) return SHAKEN_OK;  // no other members
   }
@@ -1180,6 +1223,7 @@ static void build_graph_host(shaken_ctx* c, const shaken_problem* p, HostPrep& h
                        uint32_t (&sliced)[2]) {
     int32_t dmax = 0;
     for (int64_t x = 0; x < n; ++x) dmax = std::max(dmax, ptr[x + 1] - ptr[x]);
+    c->max_deg = std::max(c->max_deg, dmax);
     std::vector<int64_t> start((size_t)dmax + 2, 0);
     for (int64_t x = 0; x < n; ++x) start[(size_t)(ptr[x + 1] - ptr[x]) + 1]++;
     for (size_t k = 1; k < start.size(); ++k) start[k] += start[k - 1];
