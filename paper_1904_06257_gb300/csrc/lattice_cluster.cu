@@ -90,6 +90,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) lattice_cluster_kernel(
   }
   cl.sync();
   const uint32_t most = (own + kClusterThreads - 1u) / kClusterThreads;  // words per thread
+  const uint32_t fwd = tid - (kClusterThreads - 64u);  // the last warps: the fewest words
   PhShared P = ph_shared(K, J.b, t0);
   uint4 W[3];  // the calls of the thread's first word
   auto call_ahead = [&](uint32_t typ) {
@@ -106,11 +107,11 @@ __global__ void __launch_bounds__(kClusterThreads, 1) lattice_cluster_kernel(
     const uint32_t* in = smem + pos * own;
     uint32_t* out = smem + (pos ^ 1u) * own;
     const uint32_t* halo = smem + 2u * own + pos * L;
-    if (track && pos == 1u && tid < 64u) {  // this block's sums to block 0
-      int* src = &part[0][0] + tid;
+    if (track && pos == 1u && fwd < 64u) {  // this block's sums to block 0
+      int* src = &part[0][0] + fwd;
       const int v = *src;
       *src = 0;
-      if (v != 0) atomicAdd(cl.map_shared_rank(all + 64u * (hs >> 1) + tid, 0), v);
+      if (v != 0) atomicAdd(cl.map_shared_rank(all + 64u * (hs >> 1) + fwd, 0), v);
     }
     if (anneal && pos == 1u) stage(t + 1u);
     // the row the neighbour needs next: dl (0) reads above, so the last row goes down
