@@ -22,7 +22,9 @@ namespace shk {
 
 constexpr int kAheadWords = 1024;  // lane words per block of lattice_ahead_kernel
 constexpr int kAheadSteps = 256;   // steps per chunk, at most
-constexpr size_t kAheadBytes = 48u << 20;  // outcome words per chunk, at most: stays in L2
+// outcome words per chunk: at most 8 MB (an allocation at the first call), or 16 steps, and at most
+// what stays in L2
+constexpr size_t kAheadBytes = 8u << 20, kAheadMost = 48u << 20;
 
 // Outcomes of NC field classes (6: 2 n + s; 4: n + s, thresholds equal within each) of every
 // lane word of a job, for step t0 + k and position p of it: out4[((job n_steps + k) 2 + p) nw + w]
@@ -115,7 +117,8 @@ __global__ void __launch_bounds__(kTile) lattice_ahead_kernel(const LatJob* __re
 
 // n_steps steps of every job, one block each, from the outcomes in out4 / out2.  DEPTH: stages
 // of the ring, one half step each; a thread loads the words it will use itself, so a stage needs
-// no barrier.  With tracking the sums of sigma_t are added per step in shared memory and
+// no barrier, and takes its first word's outcomes before the barrier that ends the half step (the
+// others' wait and loads are then off the chain).  With tracking the sums of sigma_t are added per step in shared memory and
 // turned into best energies and series after the last step.
 // Bound by the chain of a half step: barrier, neighbour loads, selects, store.
 template <int ENC, int NC, int DEPTH>
@@ -154,44 +157,65 @@ __global__ void __launch_bounds__(1024, 1) lattice_follow_kernel(
   __syncthreads();
   const uint32_t wpr = J.wpr;
   const bool pow2 = J.wpr_shift != 0xffffffffu;
+  // words of the vertical and the horizontal neighbours of lane word w (typ 0: above and left)
+  auto near = [&](uint32_t w, uint32_t typ, uint32_t& v, uint32_t& h) {
+    const uint32_t c = pow2 ? (w & (wpr - 1u)) : w % wpr;
+    if (typ == 0u) {
+      v = w >= wpr ? w - wpr : w + nw - wpr;
+      h = c == 0u ? w + wpr - 1u : w - 1u;
+    } else {
+      v = w + wpr < nw ? w + wpr : w + wpr - nw;
+      h = c + 1u == wpr ? w - c : w + 1u;
+    }
+  };
+  auto decide = [&](uint32_t S, uint32_t V, uint32_t H, const uint4& d, const uint2& e) {
+    if (NC == 4) {
+      const uint32_t c0 = V ^ H ^ S, c1 = (V & H) | (S & (V | H));
+      const uint32_t lo = (c0 & d.y) | (~c0 & d.x), hi = (c0 & d.w) | (~c0 & d.z);
+      return (c1 & hi) | (~c1 & lo);
+    }
+    const uint32_t b0 = (S & d.y) | (~S & d.x), b1 = (S & d.w) | (~S & d.z);
+    const uint32_t b2 = (S & e.y) | (~S & e.x), X = V ^ H;
+    const uint32_t m = (V & b2) | (~V & b0);
+    return (X & b1) | (~X & m);
+  };
   uint32_t s = 0;  // stage of this half step
-#pragma unroll 1
-  for (uint32_t hs = 0; hs < halves; ++hs) {
-    const uint32_t pos = hs & 1u, typ = pos ^ order;
-    const uint32_t* in = pos == 0u ? sA : sB;
-    uint32_t* out = pos == 0u ? sB : sA;
+  // the thread's first word: its neighbours' places, its spins, its outcomes of the coming half step
+  uint32_t v0, h0, v1, h1, S0 = sA[tid];
+  near(tid, order, v0, h0);
+  near(tid, order ^ 1u, v1, h1);
+  uint4 d = make_uint4(0u, 0u, 0u, 0u);
+  uint2 e = make_uint2(0u, 0u);
+  auto take_next = [&](uint32_t stage) {
+    __pipeline_wait_prior(DEPTH - 2);
+    d = ring4[stage * nw + tid];
+    if (NC == 6) e = ring2[stage * nw + tid];
+  };
+  take_next(0u);
+  auto half = [&](uint32_t hs, uint32_t pos, const uint32_t* in, uint32_t* out, uint32_t v,
+                  uint32_t h) {
+    const uint32_t typ = pos ^ order;
     const bool sums = track && pos == 0u;
-    fetch(hs + (uint32_t)DEPTH - 1u, s == 0u ? (uint32_t)DEPTH - 1u : s - 1u);
-    __pipeline_wait_prior(DEPTH - 1);
     uint32_t acc = 0u;  // +1 sites | disagreeing bonds << 16 (at most four words a thread)
-    for (uint32_t w = tid; w < nw; w += T) {
-      const uint4 d = ring4[s * nw + w];
-      const uint32_t c = pow2 ? (w & (wpr - 1u)) : w % wpr;
-      const uint32_t S = in[w];
-      uint32_t V, H;
-      if (typ == 0u) {
-        V = in[w >= wpr ? w - wpr : w + nw - wpr];
-        H = (S << 1) | (in[c == 0u ? w + wpr - 1u : w - 1u] >> 31);
-      } else {
-        V = in[w + wpr < nw ? w + wpr : w + wpr - nw];
-        H = (S >> 1) | (in[c + 1u == wpr ? w - c : w + 1u] << 31);
-      }
-      uint32_t r;
-      if (NC == 4) {
-        const uint32_t c0 = V ^ H ^ S, c1 = (V & H) | (S & (V | H));
-        const uint32_t lo = (c0 & d.y) | (~c0 & d.x), hi = (c0 & d.w) | (~c0 & d.z);
-        r = (c1 & hi) | (~c1 & lo);
-      } else {
-        const uint2 e = ring2[s * nw + w];
-        const uint32_t b0 = (S & d.y) | (~S & d.x), b1 = (S & d.w) | (~S & d.z);
-        const uint32_t b2 = (S & e.y) | (~S & e.x), X = V ^ H;
-        const uint32_t m = (V & b2) | (~V & b0);
-        r = (X & b1) | (~X & m);
-      }
+    auto one = [&](uint32_t w, uint32_t S, uint32_t V, uint32_t N, const uint4& dw,
+                   const uint2& ew) {
+      const uint32_t H = typ == 0u ? __funnelshift_l(N, S, 1) : __funnelshift_r(S, N, 1);
+      const uint32_t r = decide(S, V, H, dw, ew);
       out[w] = r;
       if (sums)
         acc += (uint32_t)__popc(S) + ((uint32_t)(__popc(S ^ V) + __popc(S ^ H)) << 16);
+      return r;
+    };
+    S0 = one(tid, S0, in[v], in[h], d, e);
+    for (uint32_t w = tid + T; w < nw; w += T) {
+      uint32_t vw, hw;
+      near(w, typ, vw, hw);
+      one(w, in[w], in[vw], in[hw], ring4[s * nw + w],
+          NC == 6 ? ring2[s * nw + w] : make_uint2(0u, 0u));
     }
+    fetch(hs + (uint32_t)DEPTH - 1u, s == 0u ? (uint32_t)DEPTH - 1u : s - 1u);
+    s = s + 1u == (uint32_t)DEPTH ? 0u : s + 1u;
+    take_next(s);
     if (sums) {
       acc = __reduce_add_sync(0xffffffffu, acc);
       if ((tid & 31u) == 0u) {
@@ -199,8 +223,12 @@ __global__ void __launch_bounds__(1024, 1) lattice_follow_kernel(
         atomicAdd(&tot[hs >> 1][1], acc >> 16);
       }
     }
-    s = s + 1u == (uint32_t)DEPTH ? 0u : s + 1u;
     __syncthreads();
+  };
+#pragma unroll 1
+  for (uint32_t hs = 0; hs < halves; hs += 2u) {
+    half(hs, 0u, sA, sB, v0, h0);
+    half(hs + 1u, 1u, sB, sA, v1, h1);
   }
   for (uint32_t w = tid; w < nw; w += T) {
     resident_store<ENC>(J, J.A, w, sA[w]);
@@ -280,6 +308,7 @@ bool lattice_ahead_faster(int nc, int n_jobs, uint32_t nw) {
 uint32_t lattice_ahead_chunk(int nc, int n_jobs, uint32_t nw, uint64_t n_steps, size_t* bytes) {
   const size_t step = (size_t)n_jobs * 2 * nw * nc * 4;
   uint64_t chunk = kAheadBytes / step;
+  if (chunk < 16) chunk = kAheadMost / step < 16 ? kAheadMost / step : 16;
   if (chunk > (uint64_t)kAheadSteps) chunk = kAheadSteps;
   if (chunk > n_steps) chunk = n_steps;
   *bytes = chunk * step;
