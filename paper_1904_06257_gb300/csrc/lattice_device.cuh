@@ -105,6 +105,32 @@ __device__ __forceinline__ LaneWord classify(uint32_t S, uint32_t V, uint32_t H,
 // differing plane, as call by call; after the twelve planes a lane is undecided
 // with probability 2^-12.
 template <bool COLL>
+__device__ __forceinline__ void decide_head3(LaneWord& L, const LatTable& tab, const PhKey& K,
+                                             const PhShared& P, uint32_t a, uint32_t half,
+                                             uint32_t& calls) {
+  const uint4 w0 = ph_call_shared(K, P, a, half);
+  const uint4 w1 = ph_call_shared(K, P, a, half + 2u);
+  const uint4 w2 = ph_call_shared(K, P, a, half + 4u);
+  calls += 3;
+  // the top twelve bits of u and T compared as a subtraction, least significant
+  // plane first (borrow lt, equality eq): two short independent chains
+  uint32_t lt = 0u, eq = 0xffffffffu;
+#pragma unroll
+  for (int j = 11; j >= 0; --j) {
+    const uint4 Wc = j >= 8 ? w2 : j >= 4 ? w1 : w0;
+    const int i = j & 3;
+    const uint32_t w = i == 0 ? Wc.x : i == 1 ? Wc.y : i == 2 ? Wc.z : Wc.w;
+    const uint32_t Pj = plane_bits<COLL>(L, plane_row<COLL>(tab, j));
+    lt = (~w & Pj) | (~w & lt) | (Pj & lt);
+    eq &= ~(w ^ Pj);
+  }
+  L.res |= L.U & ~eq & lt;
+  L.U &= eq;
+}
+
+// The same comparison from calls made before (lattice_cluster_kernel).  Not the body of
+// decide_head3: with the calls in an array the whole-run kernel took 8 % longer.
+template <bool COLL>
 __device__ __forceinline__ void decide_planes3(LaneWord& L, const LatTable& tab,
                                                const uint4 (&W)[3]) {
   // the top twelve bits of u and T compared as a subtraction, least significant
@@ -121,16 +147,6 @@ __device__ __forceinline__ void decide_planes3(LaneWord& L, const LatTable& tab,
   }
   L.res |= L.U & ~eq & lt;
   L.U &= eq;
-}
-
-template <bool COLL>
-__device__ __forceinline__ void decide_head3(LaneWord& L, const LatTable& tab, const PhKey& K,
-                                             const PhShared& P, uint32_t a, uint32_t half,
-                                             uint32_t& calls) {
-  const uint4 W[3] = {ph_call_shared(K, P, a, half), ph_call_shared(K, P, a, half + 2u),
-                      ph_call_shared(K, P, a, half + 4u)};
-  calls += 3;
-  decide_planes3<COLL>(L, tab, W);
 }
 
 // Planes 31..24 (calls 0 and 1) of the thread's WPT lane words, plane-major:
