@@ -9,8 +9,8 @@
 // all 32 planes, so the trajectory is that of the half-step kernels.
 //
 // A run that makes its own draws is a chain of three Philox calls and twelve planes a half step
-// on one SM: 1.35 us a step at L = 64, 18.5 us at L = 352.  With the draws ahead 0.47 and 3.4 us;
-// 500 recorded steps at L = 64 with state and observables read back 860 -> 363 us.
+// on one SM: 1.35 us a step at L = 64, 18.5 us at L = 352.  With the draws ahead 0.36 and 3.5 us;
+// 500 recorded steps at L = 64 with state and observables read back 860 -> 288 us.
 #include <cuda_pipeline_primitives.h>
 
 #include <cstdint>
@@ -290,11 +290,11 @@ static int follow_depth(int nc, uint32_t nw) {
   return 0;
 }
 
-// Microseconds of a step of n_jobs INT8 / PACKED lattices of nw words this way (both kernels) and
-// with the draws made by the block itself (lattice_resident_kernel, one wave of blocks).  Fitted
-// to 200 steps of sides 32 .. 352 and 1 .. 2048 replicas; both sides, L = 64: 1 replica 0.47
-// (ahead) against 1.35 us a step, 64 replicas 0.97 against 1.37, 256 replicas 2.6 against 1.7; L = 352: 1
-// replica 3.4 against 18.5, 32 replicas 9.4 against 18.6 (six classes 13.5 against 21), 152
+// Whether a step of n_jobs INT8 / PACKED lattices of nw words takes less time this way (both kernels)
+// than with the draws made by the block itself (lattice_resident_kernel, one wave of blocks).
+// Fitted to 200 steps of sides 32 .. 352 and 1 .. 2048 replicas; both sides, L = 64: 1 replica 0.36
+// (ahead) against 1.35 us a step, 64 replicas 0.87 against 1.37, 256 replicas 2.6 against 1.7; L = 352: 1
+// replica 3.5 against 18.5, 32 replicas 9.5 against 18.6 (six classes 13.7 against 21), 152
 // replicas 35 against 18.7.
 bool lattice_ahead_faster(int nc, int n_jobs, uint32_t nw) {
   if (follow_depth(nc, nw) == 0) return false;
