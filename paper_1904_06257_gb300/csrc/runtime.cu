@@ -1457,8 +1457,9 @@ static bool resident_eligible(const shaken_ctx* c, uint64_t n_steps) {
   return (uint64_t)c->L * c->L / 32 <= 4096;
 }
 
-// Field classes of different thresholds: by n + s where q = J, else by (n, s).
-static int field_classes(const shaken_ctx* c) { return c->q == c->J ? 4 : 6; }
+// Field classes of different thresholds: by n + s where q = J (and 2 J is finite: the fields of (n, s)
+// are then equal exactly), else by (n, s).
+static int field_classes(const shaken_ctx* c) { return c->q == c->J && c->J < 1e300 ? 4 : 6; }
 
 // Small MULTISPIN lattices: one thread-block cluster per group of 32 replicas, where that takes
 // less time per step than the kernels of a step on the whole GPU.  Both in microseconds per
