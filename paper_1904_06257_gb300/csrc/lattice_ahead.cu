@@ -22,9 +22,9 @@ namespace shk {
 
 constexpr int kAheadWords = 1024;  // lane words per block of lattice_ahead_kernel
 constexpr int kAheadSteps = 256;   // steps per chunk, at most
-// outcome words per chunk: at most 8 MB (an allocation at the first call), or 16 steps, and at most
-// what stays in L2
-constexpr size_t kAheadBytes = 8u << 20, kAheadMost = 48u << 20;
+// outcome words per chunk: at most 24 MB (an allocation at the first call; at 8 MB 64 replicas of L = 64
+// took 1.10 instead of 0.87 us a step), or 16 steps, and at most what stays in L2
+constexpr size_t kAheadBytes = 24u << 20, kAheadMost = 48u << 20;
 
 // Outcomes of NC field classes (6: 2 n + s; 4: n + s, thresholds equal within each) of every
 // lane word of a job, for step t0 + k and position p of it: out4[((job n_steps + k) 2 + p) nw + w]
