@@ -460,17 +460,14 @@ static size_t gcl_bytes(uint32_t n, uint64_t m, uint32_t C, int classes) {
 
 static cudaError_t gcl_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, uint32_t n,
                               uint64_t m, uint32_t C, int classes, int clusters, cudaStream_t st) {
-  const size_t bytes = gcl_bytes(n, m, C, classes);
-  const auto kernel = graph_cluster_kernel;
-  cudaError_t e =
-      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  cudaError_t e = allow_block_smem<graph_cluster_kernel>();
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    e = cudaFuncSetAttribute(graph_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
   cfg = cudaLaunchConfig_t{};
   cfg.gridDim = dim3((unsigned)clusters * C);
   cfg.blockDim = dim3(kGclThreads);
-  cfg.dynamicSmemBytes = bytes;
+  cfg.dynamicSmemBytes = gcl_bytes(n, m, C, classes);
   cfg.stream = st;
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = C;

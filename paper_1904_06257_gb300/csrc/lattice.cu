@@ -1209,6 +1209,11 @@ cudaError_t launch_lattice_obs(int enc, int wpt, const LatJob* jobs, const Tile*
 }  // namespace shk
 
 namespace shk {
+static cudaError_t allow_band_smem(int enc) {
+  return enc == kEncInt8 ? allow_block_smem<lattice_band_kernel<kEncInt8>>()
+                         : allow_block_smem<lattice_band_kernel<kEncPacked>>();
+}
+
 // Grid and shared memory of the banded kernel for an L x L lattice of wpr words
 // per row: as many co-resident blocks as fit (at most L, one row each at least).
 // Returns false when the lattice does not fit that way.
@@ -1219,6 +1224,10 @@ bool lattice_band_shape(int enc, uint32_t L, uint32_t wpr, int* grid, size_t* sm
   int max_smem = 0;
   cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   int G = sms * kBandMinBlocks;
+  if (allow_band_smem(enc) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
   for (int it = 0; it < 8; ++it) {
     if (G > (int)L) G = (int)L;
     const uint32_t rows = (L + (uint32_t)G - 1u) / (uint32_t)G + 2u;
@@ -1226,7 +1235,6 @@ bool lattice_band_shape(int enc, uint32_t L, uint32_t wpr, int* grid, size_t* sm
     if (bytes > (size_t)max_smem - sizeof(LatTable) - 64) return false;
     const void* k = enc == kEncInt8 ? (const void*)lattice_band_kernel<kEncInt8>
                                     : (const void*)lattice_band_kernel<kEncPacked>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     int o = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k, kTile, bytes);
     cudaGetLastError();
@@ -1250,7 +1258,7 @@ cudaError_t launch_lattice_band(int enc, const LatJob* jobs, int grid, size_t sm
   void* args[] = {(void*)&jobs, (void*)&xch, (void*)&bs, (void*)&t0, (void*)&n_steps};
   const void* k = enc == kEncInt8 ? (const void*)lattice_band_kernel<kEncInt8>
                                   : (const void*)lattice_band_kernel<kEncPacked>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_band_smem(enc);
   if (e != cudaSuccess) return e;
   e = cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kTile), args, smem, st);
   if (e != cudaSuccess) return e;
@@ -1266,13 +1274,11 @@ cudaError_t launch_lattice_resident(int enc, const LatJob* jobs, int n_jobs, uin
   threads = (threads + 31) / 32 * 32;
   cudaError_t e = cudaSuccess;
   if (enc == kEncInt8) {
-    e = cudaFuncSetAttribute(lattice_resident_kernel<kEncInt8>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    e = allow_block_smem<lattice_resident_kernel<kEncInt8>>();
     if (e == cudaSuccess)
       lattice_resident_kernel<kEncInt8><<<n_jobs, threads, bytes, st>>>(jobs, t0, n_steps);
   } else {
-    e = cudaFuncSetAttribute(lattice_resident_kernel<kEncPacked>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    e = allow_block_smem<lattice_resident_kernel<kEncPacked>>();
     if (e == cudaSuccess)
       lattice_resident_kernel<kEncPacked><<<n_jobs, threads, bytes, st>>>(jobs, t0, n_steps);
   }

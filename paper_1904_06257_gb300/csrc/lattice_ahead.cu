@@ -320,11 +320,9 @@ static cudaError_t follow(const LatJob* jobs, int n_jobs, uint32_t nw, uint32_t 
                           uint32_t n_steps, const uint4* out4, const uint2* out2,
                           cudaStream_t st) {
   const size_t bytes = follow_bytes(NC, nw, DEPTH);
-  const auto kernel = lattice_follow_kernel<ENC, NC, DEPTH>;
-  const cudaError_t e =
-      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  const cudaError_t e = allow_block_smem<lattice_follow_kernel<ENC, NC, DEPTH>>();
   if (e != cudaSuccess) return e;
-  kernel<<<n_jobs, nw < 1024u ? nw : 1024u, bytes, st>>>(jobs, t0, n_steps, out4, out2);
+  lattice_follow_kernel<ENC, NC, DEPTH><<<n_jobs, nw < 1024u ? nw : 1024u, bytes, st>>>(jobs, t0, n_steps, out4, out2);
   return cudaGetLastError();
 }
 

@@ -234,9 +234,7 @@ static size_t cluster_bytes(uint32_t L, uint32_t C) {
 
 static cudaError_t cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, uint32_t L,
                                   uint32_t C, int n_jobs, cudaStream_t st) {
-  const size_t bytes = cluster_bytes(L, C);
-  cudaError_t e = cudaFuncSetAttribute(lattice_cluster_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  cudaError_t e = allow_block_smem<lattice_cluster_kernel>();
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(lattice_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed,
                              1);
@@ -244,7 +242,7 @@ static cudaError_t cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* 
   cfg = cudaLaunchConfig_t{};
   cfg.gridDim = dim3((unsigned)n_jobs * C);
   cfg.blockDim = dim3(kClusterThreads);
-  cfg.dynamicSmemBytes = bytes;
+  cfg.dynamicSmemBytes = cluster_bytes(L, C);
   cfg.stream = st;
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = C;

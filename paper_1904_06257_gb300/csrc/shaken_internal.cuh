@@ -18,6 +18,7 @@
 //   * field h = (Jc * s + q * sigma) + lambda, s the integer neighbour sum.
 #pragma once
 
+#include <atomic>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -62,6 +63,28 @@ cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
+
+// Lets launches of Kernel take as much dynamic shared memory as a block can have beside its static
+// part.  The limit belongs to the function, for every thread of the process: it is raised once per
+// device and never set to one launch's size, which another thread could lower between this
+// thread's call and its launch (refused then: "invalid argument").
+template <auto Kernel>
+cudaError_t allow_block_smem() {
+  static std::atomic<uint64_t> raised{0};  // devices, by bit
+  int dev = 0, most = 0;
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaGetDevice(&dev);
+  const uint64_t bit = dev < 64 ? 1ull << dev : 0ull;
+  if (e != cudaSuccess || (raised.load() & bit) != 0ull) return e;
+  e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, Kernel);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             most - (int)fa.sharedSizeBytes);
+  if (e == cudaSuccess) raised.fetch_or(bit);
+  return e;
+}
+
 constexpr int kWordsPerThread = 4;                   // lattice lane words per thread and tile
 constexpr int kLatTile = kTile * kWordsPerThread;    // lattice lane words per tile
 constexpr int kLatMinBlocks = 3;                     // resident blocks per SM of the half-step kernel
