@@ -36,6 +36,8 @@ namespace shk {
 
 namespace cg = cooperative_groups;
 
+cudaError_t launch_advance(CtxDev* const*, int, uint32_t, cudaStream_t);
+
 constexpr int kGclThreads = 512;
 constexpr int kGclWarps = kGclThreads / 32;
 constexpr int kAheadThreads = 256;  // of graph_ahead_kernel
@@ -432,14 +434,6 @@ __global__ void __launch_bounds__(kGclThreads, 1) graph_cluster_kernel(
   }
 }
 
-// The step counters of contexts whose whole run went through graph_cluster_kernel.
-__global__ void advance_kernel(CtxDev* const* __restrict__ ctxs, int n, uint32_t steps) {
-  const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x);
-  if (i >= n) return;
-  CtxDev* cd = ctxs[i];
-  if (cd->step < cd->t_end) cd->step += min(steps, cd->t_end - cd->step);
-}
-
 // Padded column words of a block and direction.  Passes ascend by degree, so 32 x the largest
 // degree of a pass is at most the edges of the next one (if that is whole), and the edges of
 // every C-th pass are at most m / C and one pass; the last two passes have no whole next
@@ -535,8 +529,7 @@ cudaError_t launch_graph_cluster(const GraphJob* jobs, const uint32_t* off, int 
     e = cudaLaunchKernelEx(&cfg, graph_cluster_kernel, jobs, off, steps,
                            gcl_col_words(m, (uint32_t)C), ptot, stride, (const uint32_t*)out);
   if (e != cudaSuccess) return e;
-  advance_kernel<<<(n_ctx + 127) / 128, 128, 0, st>>>(ctxs, n_ctx, steps);
-  return cudaGetLastError();
+  return launch_advance(ctxs, n_ctx, steps, st);
 }
 
 }  // namespace shk

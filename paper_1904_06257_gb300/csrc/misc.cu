@@ -138,9 +138,24 @@ cudaError_t launch_member_copy(int what, const MemberDev* m, int n, void* buf,
   return cudaGetLastError();
 }
 
+// The step counters of contexts whose whole run went through a kernel that leaves them (the cluster
+// kernels): on the stream, behind the run.
+__global__ void advance_kernel(CtxDev* const* __restrict__ ctxs, int n, uint32_t steps) {
+  const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  if (i >= n) return;
+  CtxDev* cd = ctxs[i];
+  if (cd->step < cd->t_end) cd->step += min(steps, cd->t_end - cd->step);
+}
+
 cudaError_t launch_epilogue(CtxDev* const* ctxs, int n, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   return launch_dependent(epilogue_kernel, dim3(n), dim3(256), 0, st, ctxs, n);
+}
+
+cudaError_t launch_advance(CtxDev* const* ctxs, int n, uint32_t steps, cudaStream_t st) {
+  if (n <= 0) return cudaSuccess;
+  advance_kernel<<<(n + 127) / 128, 128, 0, st>>>(ctxs, n, steps);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_philox(uint64_t seed, const uint32_t* ctr, uint32_t* out, int64_t n,

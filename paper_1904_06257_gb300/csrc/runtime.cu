@@ -59,6 +59,7 @@ cudaError_t launch_graph_obs_group(bool, const GraphJob*, const Tile*, int, int,
 cudaError_t launch_graph_fields(const GraphJob*, const Tile*, int, uint32_t, float*,
                                 cudaStream_t);
 cudaError_t launch_epilogue(CtxDev* const*, int, cudaStream_t);
+cudaError_t launch_advance(CtxDev* const*, int, uint32_t, cudaStream_t);
 cudaError_t launch_member_copy(int, const shk::MemberDev*, int, void*, unsigned long long,
                                cudaStream_t);
 bool lattice_band_shape(int, uint32_t, uint32_t, int*, size_t*);
@@ -1531,8 +1532,11 @@ static shaken_status run_cluster(shaken_ctx* c, uint64_t n_steps) {
     c->launches++;
     done += chunk;
   }
+  // the device step counter follows on the stream: the call returns before the run is done
+  CU(shk::launch_advance(c->solo.ctxlist.as<CtxDev*>(), 1, (uint32_t)n_steps, st));
+  c->launches++;
   c->host_step += n_steps;
-  return push_cd(c);
+  return SHAKEN_OK;
 }
 
 // Mid-size single lattices (INT8/PACKED, one replica, beyond the resident size)
