@@ -47,8 +47,6 @@ __device__ __forceinline__ void add_plane(uint32_t (&p)[N], uint32_t x, int b0) 
   }
 }
 
-constexpr uint32_t kClusterSteps = 128;  // steps per chunk, at most: their sums stay in shared memory
-
 __global__ void __launch_bounds__(kClusterThreads, 1) lattice_cluster_kernel(
     const LatJob* __restrict__ jobs, uint32_t t0, uint32_t n_steps) {
   extern __shared__ __align__(16) uint32_t smem[];
@@ -284,17 +282,15 @@ int lattice_cluster_shape(uint32_t L, int n_jobs, double* us) {
   return best;
 }
 
-// n_steps of every group, a launch per chunk.
+// n_steps of every group, at most kClusterSteps.
 cudaError_t launch_lattice_cluster(const LatJob* jobs, int n_jobs, uint32_t L, int C, uint32_t t0,
                                    uint32_t n_steps, cudaStream_t st) {
   if (n_jobs <= 0 || n_steps == 0) return cudaSuccess;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
-  cudaError_t e = cluster_config(cfg, attr, L, (uint32_t)C, n_jobs, st);
-  for (uint32_t k = 0; k < n_steps && e == cudaSuccess; k += kClusterSteps)
-    e = cudaLaunchKernelEx(&cfg, lattice_cluster_kernel, jobs, t0 + k,
-                           n_steps - k < kClusterSteps ? n_steps - k : kClusterSteps);
-  return e;
+  const cudaError_t e = cluster_config(cfg, attr, L, (uint32_t)C, n_jobs, st);
+  return e != cudaSuccess ? e
+                          : cudaLaunchKernelEx(&cfg, lattice_cluster_kernel, jobs, t0, n_steps);
 }
 
 }  // namespace shk

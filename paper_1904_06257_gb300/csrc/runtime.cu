@@ -1526,7 +1526,7 @@ static shaken_status run_cluster(shaken_ctx* c, uint64_t n_steps) {
   const Family& F = *c->solo.fams[0];
   uint64_t done = 0;
   while (done < n_steps) {
-    const uint64_t chunk = std::min<uint64_t>(n_steps - done, 1u << 16);
+    const uint64_t chunk = std::min<uint64_t>(n_steps - done, shk::kClusterSteps);
     CU(shk::launch_lattice_cluster(F.jobs.as<LatJob>(), c->R / 32, (uint32_t)c->L, c->cluster,
                                    (uint32_t)(c->host_step + done), (uint32_t)chunk, st));
     c->launches++;

@@ -36,6 +36,8 @@ constexpr int kSlicedTile = 128;  // threads per block (and tile) of the bit-sli
 constexpr int kSlicedShapes = 5;
 constexpr int kSlicedWords[kSlicedShapes] = {1, 2, 3, 4, 4};
 constexpr bool kSlicedVec[kSlicedShapes] = {true, true, false, true, false};
+// Steps of a launch of the MULTISPIN cluster kernel, at most: their sums stay in shared memory.
+constexpr uint32_t kClusterSteps = 128;
 
 // ---------------------------------------------------------------- dependent launches
 // The kernels of a step (half steps, observables, epilogue) are launched with

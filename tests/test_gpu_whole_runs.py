@@ -35,3 +35,12 @@ def test_multispin_step_returns_before_the_gpu_is_done(S, L, R, track):
         S.shaken_free(c)
     for a, b in zip(*ends):
         assert np.array_equal(a, b)
+
+
+def test_launch_count_of_a_cluster_run(S):
+    """300 steps of a small MULTISPIN lattice: three launches of at most 128 steps and one that moves the step on."""
+    c = S.shaken_init(lattice_problem(S, S.MULTISPIN, 64, 32, 0.5), 5)
+    before = S.shaken_launch_count(c)
+    S.shaken_step(c, 300)
+    assert S.shaken_launch_count(c) - before == 4
+    S.shaken_free(c)
