@@ -147,6 +147,10 @@ void shaken_free(shaken_ctx* ctx);
  * as before it).  MULTISPIN lattices of small sides (n >= 4) and small +-1 graphs
  * also run in whole chunks, each group of 32 replicas in one thread-block
  * cluster, and stay asynchronous.  Every path gives the same trajectory.
+ * If a CUDA call fails in the middle of a run of any length (this call, an
+ * anneal, a recorded run, a batch step), its error is returned with the whole
+ * steps issued before it applied and counted (shaken_get_step; in a batch each
+ * member's own count), and the context goes on from there.
  * E_STATE if the context is owned by a batch. */
 shaken_status shaken_step(shaken_ctx* ctx, uint64_t n_steps);
 
@@ -246,6 +250,12 @@ shaken_status shaken_debug_band_stall(shaken_ctx* ctx);
  * all arrived, the call then either succeeds with the chunk applied or returns
  * SHAKEN_E_TIMEOUT with the state as before the chunk -- never a mixture. */
 shaken_status shaken_debug_band_hurry(shaken_ctx* ctx, int block);
+
+/* Diagnostics for the failure path of runs in chunks: the (after + 1)-th chunk of
+ * steps from now on -- a launch of a whole run, a replay of captured steps, or a
+ * step of half-step launches -- of this context (of its batch, for a member) is
+ * not issued, and the call returns SHAKEN_E_CUDA as if the launch had been refused. */
+shaken_status shaken_debug_refuse_chunk(shaken_ctx* ctx, int after);
 
 /* Number of kernel launches this context has issued (all kinds). */
 shaken_status shaken_launch_count(shaken_ctx* ctx, uint64_t* count);

@@ -519,12 +519,16 @@ cudaError_t launch_graph_cluster(const GraphJob* jobs, const uint32_t* off, int 
   uint32_t* const out = static_cast<uint32_t*>(work);
   uint2* const tab = reinterpret_cast<uint2*>(out + (size_t)2 * steps * ptot * stride);
   graph_thresholds_kernel<<<(unsigned)clusters * steps, 128, 0, st>>>(jobs, steps, tab);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
   const uint32_t per = ((n + 31u) / 32u + kAheadThreads / 32 - 1u) / (kAheadThreads / 32);
   graph_ahead_kernel<<<(unsigned)clusters * steps * 2u * per, kAheadThreads, 0, st>>>(
       jobs, off, steps, per, ptot, stride, tab, out);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
-  cudaError_t e = gcl_config(cfg, attr, n, m, (uint32_t)C, classes, clusters, st);
+  e = gcl_config(cfg, attr, n, m, (uint32_t)C, classes, clusters, st);
   if (e == cudaSuccess)
     e = cudaLaunchKernelEx(&cfg, graph_cluster_kernel, jobs, off, steps,
                            gcl_col_words(m, (uint32_t)C), ptot, stride, (const uint32_t*)out);

@@ -208,6 +208,7 @@ struct Plan {
   int graph_steps = 0;
   uint64_t graph_launches = 0;
   bool dirty = true;
+  int refuse = -1;  // diagnostics: chunks of steps until one is refused (-1: none is)
   bool autotune = true;  // pick the lattice tile shape by timing trial launches
   int pinned[3][2] = {{0, 0}, {0, 0}, {0, 0}};  // per lattice encoding: (wpt, bps) set by the caller
   int blocks_per_sm = 8;
@@ -958,10 +959,24 @@ static shaken_status plan_step_launch(Plan& P, cudaStream_t st, uint64_t* nl,
 
 static constexpr int kGraphChunk = 32;
 
+// Full steps that a run of a plan has issued: members in clusters, and the others.
+struct Issued {
+  uint64_t clusters = 0, rest = 0;
+  uint64_t of(const Plan& P, const shaken_ctx* c) const {
+    return c->kind == SHAKEN_GRAPH && P.cl_clusters > 0 ? clusters : rest;
+  }
+};
+
+// Before each chunk of a run (a launch sequence that moves the step counter once).
+static shaken_status may_issue(Plan& P) {
+  if (P.refuse < 0 || P.refuse-- > 0) return SHAKEN_OK;
+  return fail(SHAKEN_E_CUDA, "diagnostics: chunk refused");
+}
+
+// `issued` tells how far the members' states and device step counters have moved, also on error.
 static shaken_status plan_run(Plan& P, cudaStream_t st, uint64_t n_steps, bool use_graph,
-                              uint64_t* nl) {
+                              uint64_t* nl, Issued* issued) {
   if (P.dirty) TRY(build_plan(P, st));
-  uint64_t done = 0;
   if (P.cl_clusters > 0) {
     const size_t work =
         shk::graph_cluster_step_bytes(P.cl_classes, P.cl_clusters, P.cl_passes) *
@@ -975,13 +990,15 @@ static shaken_status plan_run(Plan& P, cudaStream_t st, uint64_t n_steps, bool u
     }
   }
   if (P.cl_clusters > 0) {
-    for (uint64_t k = 0; k < n_steps; k += P.cl_chunk) {
+    while (issued->clusters < n_steps) {
+      const uint64_t chunk = std::min<uint64_t>(n_steps - issued->clusters, P.cl_chunk);
+      TRY(may_issue(P));
       CU(shk::launch_graph_cluster(P.cl_jobs.as<GraphJob>(), P.cl_off.as<uint32_t>(), P.cl_clusters,
                                    P.cl_n, P.cl_m, P.cl_classes, P.cl_passes, P.cl_blocks,
-                                   P.cl_ctx.as<CtxDev*>(), P.cl_n_ctx,
-                                   (uint32_t)std::min<uint64_t>(n_steps - k, P.cl_chunk),
+                                   P.cl_ctx.as<CtxDev*>(), P.cl_n_ctx, (uint32_t)chunk,
                                    P.cl_work.p, st));
       *nl += 4;
+      issued->clusters += chunk;
     }
     if (P.n_ctx == 0) return SHAKEN_OK;  // no other members
   }
@@ -1020,13 +1037,23 @@ static shaken_status plan_run(Plan& P, cudaStream_t st, uint64_t n_steps, bool u
       P.graph_steps = kGraphChunk;
       P.graph_launches = cnt;
     }
-    while (n_steps - done >= (uint64_t)P.graph_steps) {
+    while (n_steps - issued->rest >= (uint64_t)P.graph_steps) {
+      TRY(may_issue(P));
       CU(cudaGraphLaunch(P.gexec, st));
       *nl += P.graph_launches;
-      done += (uint64_t)P.graph_steps;
+      issued->rest += (uint64_t)P.graph_steps;
     }
   }
-  for (; done < n_steps; ++done) TRY(plan_step_launch(P, st, nl));
+  for (; issued->rest < n_steps; ++issued->rest) {
+    shaken_status s = may_issue(P);
+    if (s == SHAKEN_OK) s = plan_step_launch(P, st, nl);
+    if (s != SHAKEN_OK) {  // the step is not taken: nor are its sums, if its first half added some
+      for (shaken_ctx* c : P.members)
+        cudaMemsetAsync(c->step_sums.p, 0, c->step_sums.bytes, st);
+      cudaGetLastError();
+      return s;
+    }
+  }
   return SHAKEN_OK;
 }
 
@@ -1501,11 +1528,12 @@ static shaken_status run_resident(shaken_ctx* c, uint64_t n_steps) {
   uint32_t ahead = 0;
   if (shk::lattice_ahead_faster(nc, c->R, words))
     ahead = ahead_chunk(c, nc, c->R, words, n_steps);
-  uint64_t done = 0;
-  while (done < n_steps) {
+  const uint64_t end = c->host_step + n_steps;
+  auto next = [&]() -> shaken_status {  // a chunk
     const uint32_t chunk =
-        (uint32_t)std::min<uint64_t>(n_steps - done, ahead > 0 ? ahead : 1u << 16);
-    const uint32_t t = (uint32_t)(c->host_step + done);
+        (uint32_t)std::min<uint64_t>(end - c->host_step, ahead > 0 ? ahead : 1u << 16);
+    const uint32_t t = (uint32_t)c->host_step;
+    TRY(may_issue(c->solo));
     if (ahead > 0) {
       CU(shk::launch_lattice_ahead(nc, F.jobs.as<LatJob>(), c->R, words, t, chunk, c->ahead.p, st));
       CU(shk::launch_lattice_follow(F.enc, nc, F.jobs.as<LatJob>(), c->R, words, t, chunk,
@@ -1514,10 +1542,13 @@ static shaken_status run_resident(shaken_ctx* c, uint64_t n_steps) {
       CU(shk::launch_lattice_resident(F.enc, F.jobs.as<LatJob>(), c->R, words, t, chunk, st));
     }
     c->launches += ahead > 0 ? 2 : 1;
-    done += chunk;
-  }
-  c->host_step += n_steps;
-  return push_cd(c);  // the device step counter follows the host's
+    c->host_step += chunk;
+    return SHAKEN_OK;
+  };
+  shaken_status s = SHAKEN_OK;
+  while (s == SHAKEN_OK && c->host_step < end) s = next();
+  const shaken_status sp = push_cd(c);  // the device step counter follows the host's
+  return s != SHAKEN_OK ? s : sp;
 }
 
 static shaken_status run_cluster(shaken_ctx* c, uint64_t n_steps) {
@@ -1525,18 +1556,23 @@ static shaken_status run_cluster(shaken_ctx* c, uint64_t n_steps) {
   if (c->solo.dirty) TRY(build_plan(c->solo, st));
   const Family& F = *c->solo.fams[0];
   uint64_t done = 0;
-  while (done < n_steps) {
+  auto next = [&]() -> shaken_status {  // a chunk
     const uint64_t chunk = std::min<uint64_t>(n_steps - done, shk::kClusterSteps);
+    TRY(may_issue(c->solo));
     CU(shk::launch_lattice_cluster(F.jobs.as<LatJob>(), c->R / 32, (uint32_t)c->L, c->cluster,
                                    (uint32_t)(c->host_step + done), (uint32_t)chunk, st));
     c->launches++;
     done += chunk;
-  }
+    return SHAKEN_OK;
+  };
+  shaken_status s = SHAKEN_OK;
+  while (s == SHAKEN_OK && done < n_steps) s = next();
+  c->host_step += done;
+  if (done == 0) return s;
   // the device step counter follows on the stream: the call returns before the run is done
-  CU(shk::launch_advance(c->solo.ctxlist.as<CtxDev*>(), 1, (uint32_t)n_steps, st));
+  CU(shk::launch_advance(c->solo.ctxlist.as<CtxDev*>(), 1, (uint32_t)done, st));
   c->launches++;
-  c->host_step += n_steps;
-  return SHAKEN_OK;
+  return s;
 }
 
 // Mid-size single lattices (INT8/PACKED, one replica, beyond the resident size)
@@ -1560,9 +1596,10 @@ static shaken_status run_band(shaken_ctx* c, uint64_t n_steps, int grid, size_t 
   const size_t xbytes = (size_t)2 * grid * wpr * sizeof(uint64_t);
   if (c->band_xch.p == nullptr || c->band_xch.bytes < xbytes) TRY(c->band_xch.alloc(xbytes));
   if (c->band_sync.p == nullptr) TRY(c->band_sync.alloc(sizeof(shk::BandSync)));
-  uint64_t done = 0;
-  while (done < n_steps) {
-    const uint64_t chunk = std::min<uint64_t>(n_steps - done, 1u << 16);
+  const uint64_t end = c->host_step + n_steps;
+  auto next = [&]() -> shaken_status {  // a chunk
+    const uint64_t chunk = std::min<uint64_t>(end - c->host_step, 1u << 16);
+    TRY(may_issue(c->solo));
     shk::BandSync h0{};
     h0.hurry = c->band_hurry >= 0 ? (unsigned)c->band_hurry : ~0u;
     if (c->band_stall) h0.count = (unsigned)grid;  // no block is ever the last to arrive
@@ -1577,17 +1614,16 @@ static shaken_status run_band(shaken_ctx* c, uint64_t n_steps, int grid, size_t 
     shk::BandSync h{};
     CU(cudaMemcpyAsync(&h, c->band_sync.p, sizeof(h), cudaMemcpyDeviceToHost, st));
     CU(cudaStreamSynchronize(st));
-    if (h.commit != 1u) {
-      // the run was aborted before any block wrote the chunk back: the state is the
-      // one before the chunk, and the step counter says so
-      TRY(push_cd(c));
+    if (h.commit != 1u)  // aborted before any block wrote the chunk back: the state is the one before it
       return fail(SHAKEN_E_TIMEOUT,
                   "banded run: a grid barrier wait ran out; the chunk was not applied");
-    }
     c->host_step += chunk;
-    done += chunk;
-  }
-  return push_cd(c);  // the device step counter follows the host's
+    return SHAKEN_OK;
+  };
+  shaken_status s = SHAKEN_OK;
+  while (s == SHAKEN_OK && c->host_step < end) s = next();
+  const shaken_status sp = push_cd(c);  // the device step counter follows the host's
+  return s != SHAKEN_OK ? s : sp;
 }
 
 // INT8 runs of the half-step kernels go through the PACKED ones on a bit copy of the state: the draws
@@ -1602,20 +1638,21 @@ static bool bits_eligible(const shaken_ctx* c, uint64_t n_steps) {
   return (double)n_steps * 3.0e-5 * words > 8.0 + 1.6e-5 * words;
 }
 
-static shaken_status run_bits(shaken_ctx* c, uint64_t n_steps, uint64_t* nl) {
+static shaken_status run_bits(shaken_ctx* c, uint64_t n_steps, uint64_t* nl, Issued* issued) {
   cudaStream_t st = c->stream;
   if (c->solo.dirty) TRY(build_plan(c->solo, st));
   const size_t words = c->spin_bytes / 32;
   uint32_t* w = c->bits.as<uint32_t>();
   CU(shk::launch_bits(1, c->A.as<uint4>(), w, nullptr, words, st));
   std::swap(c->solo.fams, c->solo.bits);
-  const shaken_status s = plan_run(c->solo, st, n_steps, n_steps >= 64, nl);
+  const shaken_status s = plan_run(c->solo, st, n_steps, n_steps >= 64, nl, issued);
   std::swap(c->solo.fams, c->solo.bits);
-  if (s != SHAKEN_OK) return s;
+  *nl += 1;
+  if (issued->rest == 0) return s;  // no step taken: the bytes are the state
   CU(shk::launch_bits(0, nullptr, w, c->A.as<uint4>(), words, st));
   CU(shk::launch_bits(0, nullptr, w + words, c->B.as<uint4>(), words, st));
-  *nl += 3;
-  return SHAKEN_OK;
+  *nl += 2;
+  return s;
 }
 
 static shaken_status solo_run(shaken_ctx* ctx, uint64_t n_steps) {
@@ -1625,17 +1662,18 @@ static shaken_status solo_run(shaken_ctx* ctx, uint64_t n_steps) {
   size_t smem = 0;
   if (band_eligible(ctx, n_steps, &grid, &smem)) return run_band(ctx, n_steps, grid, smem);
   uint64_t nl = 0;
+  Issued issued;
   bool bits = bits_eligible(ctx, n_steps);
   if (bits && ctx->bits.p == nullptr) {  // no memory for the copy: on the bytes
     bits = ctx->bits.alloc(ctx->spin_bytes / 4) == SHAKEN_OK;
     if (bits) ctx->solo.invalidate();
   }
-  const shaken_status s = bits ? run_bits(ctx, n_steps, &nl)
-                               : plan_run(ctx->solo, ctx->stream, n_steps, n_steps >= 64, &nl);
+  const shaken_status s =
+      bits ? run_bits(ctx, n_steps, &nl, &issued)
+           : plan_run(ctx->solo, ctx->stream, n_steps, n_steps >= 64, &nl, &issued);
   ctx->launches += nl;
-  if (s != SHAKEN_OK) return s;
-  ctx->host_step += n_steps;
-  return SHAKEN_OK;
+  ctx->host_step += issued.of(ctx->solo, ctx);
+  return s;
 }
 
 shaken_status shaken_step(shaken_ctx* ctx, uint64_t n_steps) {
@@ -1702,8 +1740,8 @@ shaken_status shaken_anneal(shaken_ctx* ctx, const double* beta_schedule, uint64
   if (n_steps == 0) return SHAKEN_OK;
   TRY(check_steps(ctx, n_steps));
   TRY(begin_anneal(ctx, beta_schedule, n_steps));
-  TRY(solo_run(ctx, n_steps));
-  return end_anneal(ctx);
+  const shaken_status s = solo_run(ctx, n_steps), se = end_anneal(ctx);
+  return s != SHAKEN_OK ? s : se;
 }
 
 static constexpr size_t kSeriesKept = 8u << 20;  // bytes of a series buffer kept for the next run
@@ -1723,21 +1761,25 @@ shaken_status shaken_step_record(shaken_ctx* ctx, uint64_t n_steps, double* mag,
   ctx->hcd.series_H = ctx->series_H.as<double>();
   ctx->hcd.tracking = 1u;
   ctx->solo.invalidate();
-  TRY(push_cd(ctx));
-  TRY(solo_run(ctx, n_steps));
-  if (mag) CU(cudaMemcpyAsync(mag, ctx->series_m.p, bytes, cudaMemcpyDeviceToHost, ctx->stream));
-  if (energy)
-    CU(cudaMemcpyAsync(energy, ctx->series_H.p, bytes, cudaMemcpyDeviceToHost, ctx->stream));
-  CU(cudaStreamSynchronize(ctx->stream));
+  auto run = [&]() -> shaken_status {
+    TRY(push_cd(ctx));
+    TRY(solo_run(ctx, n_steps));
+    if (mag) CU(cudaMemcpyAsync(mag, ctx->series_m.p, bytes, cudaMemcpyDeviceToHost, ctx->stream));
+    if (energy)
+      CU(cudaMemcpyAsync(energy, ctx->series_H.p, bytes, cudaMemcpyDeviceToHost, ctx->stream));
+    CU(cudaStreamSynchronize(ctx->stream));
+    return SHAKEN_OK;
+  };
+  const shaken_status s = run();
   ctx->hcd.record = 0u;
   ctx->hcd.series_m = nullptr;
   ctx->hcd.series_H = nullptr;
   ctx->hcd.tracking = ctx->tracking ? 1u : 0u;
   ctx->solo.invalidate();
-  TRY(push_cd(ctx));
+  const shaken_status sp = push_cd(ctx);
   if (ctx->series_m.bytes > kSeriesKept) ctx->series_m.release();
   if (ctx->series_H.bytes > kSeriesKept) ctx->series_H.release();
-  return SHAKEN_OK;
+  return s != SHAKEN_OK ? s : sp;
 }
 
 // Observables in two parts: the device sums of a context's replicas are
@@ -2134,6 +2176,12 @@ shaken_status shaken_debug_exact_always(shaken_ctx* ctx, int on) {
   return SHAKEN_OK;
 }
 
+shaken_status shaken_debug_refuse_chunk(shaken_ctx* ctx, int after) {
+  if (!ctx || after < 0) return fail(SHAKEN_E_INVAL, "bad argument");
+  (ctx->owner ? ctx->owner->plan : ctx->solo).refuse = after;
+  return SHAKEN_OK;
+}
+
 shaken_status shaken_debug_band_hurry(shaken_ctx* ctx, int block) {
   if (!ctx || block < 0) return fail(SHAKEN_E_INVAL, "bad argument");
   ctx->band_hurry = block;
@@ -2181,11 +2229,11 @@ shaken_status shaken_batch_step(shaken_batch* b, uint64_t n_steps, int use_graph
   if (b->plan.members.empty() || n_steps == 0) return SHAKEN_OK;
   for (shaken_ctx* c : b->plan.members) TRY(check_steps(c, n_steps));
   uint64_t nl = 0;
-  shaken_status s = plan_run(b->plan, b->stream, n_steps, use_graph != 0, &nl);
+  Issued issued;
+  const shaken_status s = plan_run(b->plan, b->stream, n_steps, use_graph != 0, &nl, &issued);
   b->launches += nl;
-  if (s != SHAKEN_OK) return s;
-  for (shaken_ctx* c : b->plan.members) c->host_step += n_steps;
-  return SHAKEN_OK;
+  for (shaken_ctx* c : b->plan.members) c->host_step += issued.of(b->plan, c);
+  return s;
 }
 
 shaken_status shaken_batch_sync(shaken_batch* b) {
@@ -2514,7 +2562,8 @@ static void server_loop(shaken_server* s) {
     uint64_t chunk = s->chunk;
     lk.unlock();
     uint64_t nl = 0;
-    shaken_status st = plan_run(s->batch.plan, s->stream, chunk, true, &nl);
+    Issued issued;
+    shaken_status st = plan_run(s->batch.plan, s->stream, chunk, true, &nl, &issued);
     if (st == SHAKEN_OK) {
       cudaError_t e = cudaStreamSynchronize(s->stream);
       if (e != cudaSuccess) st = fail(SHAKEN_E_CUDA, cudaGetErrorString(e));

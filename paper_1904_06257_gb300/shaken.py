@@ -83,6 +83,7 @@ def _load():
         "shaken_debug_exact_always": [vp, ctypes.c_int],
         "shaken_debug_band_stall": [vp],
         "shaken_debug_band_hurry": [vp, ctypes.c_int],
+        "shaken_debug_refuse_chunk": [vp, ctypes.c_int],
         "shaken_launch_count": [vp, ctypes.POINTER(u64)],
         "shaken_sync": [vp],
         "shaken_batch_create": [ctypes.POINTER(vp), vp],
@@ -298,6 +299,11 @@ def shaken_debug_band_stall(ctx):
 
 def shaken_debug_band_hurry(ctx, block: int):
     _check(_lib.shaken_debug_band_hurry(ctx, int(block)))
+
+
+def shaken_debug_refuse_chunk(ctx, after: int):
+    """The (after + 1)-th chunk of steps from now on is refused (failure-path test)."""
+    _check(_lib.shaken_debug_refuse_chunk(ctx, int(after)))
 
 
 def shaken_launch_count(ctx) -> int:
