@@ -192,19 +192,23 @@ struct Plan {
   std::vector<shaken_ctx*> members;
   std::vector<std::unique_ptr<Family>> fams;
   std::vector<std::unique_ptr<Family>> bits;  // INT8 lattice: its half steps on the bit copy
-  DevMem ctxlist;
-  int n_ctx = 0;
-  // graph members stepped in whole runs, one cluster of cl_blocks blocks per group (cl_clusters
-  // of them, cl_n_ctx members of at most cl_n vertices and cl_m edges); the others: ctxlist
-  // vertices have at most cl_classes classes; cl_off: a group's first 32-vertex pass among
-  // cl_passes; cl_work: the outcome words of up to cl_chunk steps
-  DevMem cl_jobs, cl_ctx, cl_off, cl_work;
+  DevMem ctxlist;  // the members that never go in clusters (n_rest) first
+  int n_ctx = 0, n_rest = 0;
+  // graph members that long enough calls step in whole runs (clusters_pay), one cluster of
+  // cl_blocks blocks per group (cl_clusters of them, cl_n_ctx members of at most cl_n vertices and
+  // cl_m edges); vertices have at most cl_classes classes; cl_off: a group's first 32-vertex pass
+  // among cl_passes; cl_work: the outcome words of up to cl_chunk steps.  Microseconds of a step's
+  // chain and outcome words, a chunk's loads, a call; of a step of the half-step kernels.
+  DevMem cl_jobs, cl_off, cl_work;
   int cl_clusters = 0, cl_blocks = 0, cl_n_ctx = 0, cl_classes = 0;
   uint32_t cl_n = 0, cl_passes = 0, cl_chunk = 0;
   uint64_t cl_m = 0;
+  double cl_chain_us = 0.0, cl_ahead_us = 0.0, cl_chunk_us = 0.0, cl_call_us = 0.0, half_us = 0.0;
   bool cl_refused = false;  // no memory for cl_work
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
+  int graph_what = 0;  // what the captured steps are of (plan_run)
+  bool on_bits = false;  // fams and bits are exchanged (run_bits)
   int graph_steps = 0;
   uint64_t graph_launches = 0;
   bool dirty = true;
@@ -577,19 +581,19 @@ static shaken_status choose_lattice_shape(const Plan& P, int enc, const std::vec
   return SHAKEN_OK;
 }
 
-// Whether the graph members of a plan are stepped in whole runs by graph_cluster_kernel: +-1
-// couplings, one lambda, every vertex and half step within the bit-sliced kernel, and less
-// time per step than the half-step kernels and the epilogue.  The run takes its chain
-// (shk::graph_cluster_shape), the outcome words made ahead (29 ns per 1000 words and class) and a
-// chunk's launches and loads; the half-step kernels 14.3 us and 40 ns per 1000 words, tracked
-// 18 us and 60 ns.  Measured on both sides of the line, mean degree 8, 200 annealed steps:
-// n = 8000, four groups 11.2 (cluster) against 21.2 us a step, eight groups 19.5 against 24.1;
-// 100 plain steps: 10.3 against 16.3, eight groups 17.9 against 17.6.  (With a lambda per vertex
-// the thresholds would be each vertex's own.)  Sets the plan's cluster size.
-// Bytes of outcome words, at most: they stay in L2.  (Chunks of 64 steps instead of what fits, up to 256:
-// 500 annealed steps of n = 2000 2.17 -> 2.42 ms, and the first run no shorter.)
+// Bytes of a chunk's outcome words, at most: they stay in L2.  (Chunks of 64 steps instead of what
+// fits, up to 256: 500 annealed steps of n = 2000 2.17 -> 2.42 ms, and the first run no shorter.)
 static constexpr size_t kClusterWork = 64u << 20;
 
+// Whether the graph members of a plan can be stepped in whole runs by graph_cluster_kernel -- +-1
+// couplings, one lambda, every vertex and half step within the bit-sliced kernel -- and long runs
+// take less time per step that way than with the half-step kernels and the epilogue.  The run
+// takes its chain (shk::graph_cluster_shape), the outcome words made ahead (29 ns per 1000 words
+// and class) and a chunk's launches and loads; the half-step kernels 14.3 us and 40 ns per 1000
+// words, tracked 18 us and 60 ns.  Measured on both sides of the line, mean degree 8, 200 annealed
+// steps: n = 8000, four groups 11.2 (cluster) against 21.2 us a step, eight groups 19.5 against
+// 24.1; 100 plain steps: 10.3 against 16.3, eight groups 17.9 against 17.6.  (With a lambda per
+// vertex the thresholds would be each vertex's own.)  Sets the plan's cluster size and times.
 static void choose_clusters(Plan& P) {
   P.cl_clusters = P.cl_blocks = P.cl_n_ctx = 0;
   P.cl_n = 0;
@@ -624,8 +628,12 @@ static void choose_clusters(Plan& P) {
   const size_t step = shk::graph_cluster_step_bytes(classes, clusters, (uint32_t)passes);
   const uint32_t chunk = (uint32_t)std::min<size_t>(kClusterWork / step, 256);
   if (blocks == 0 || chunk == 0) return;
-  us += 2.9e-5 * outcomes + (8.0 + 6e-4 * most) / chunk;
-  if (us >= (tracked ? 18.0 + 6e-5 * words : 14.3 + 4e-5 * words)) return;
+  P.cl_chain_us = us;
+  P.cl_ahead_us = 2.9e-5 * outcomes;
+  P.cl_chunk_us = 8.0 + 6e-4 * most;
+  P.cl_call_us = 1.4e-3 * most;
+  P.half_us = tracked ? 18.0 + 6e-5 * words : 14.3 + 4e-5 * words;
+  if (P.cl_chain_us + P.cl_ahead_us + P.cl_chunk_us / chunk >= P.half_us) return;
   P.cl_classes = classes;
   P.cl_passes = (uint32_t)passes;
   P.cl_chunk = chunk;
@@ -634,6 +642,18 @@ static void choose_clusters(Plan& P) {
   P.cl_n_ctx = members;
   P.cl_n = most;
   P.cl_m = edges;
+}
+
+// Whether a call of n steps is long enough for clusters: it also pays for the set-up of its first
+// chunk, however few steps follow, and outcome words of few steps take 25 us (a launch that does not
+// fill the GPU).  Microseconds a step in calls of 1, 3, 4 and 8, half-step kernels against
+// clusters: n = 2000, one group 14.1 against 36.1, 14.3, 11.5 and 7.3; n = 8000, four groups 16.4
+// against 52.6, 21.7, 17.9 and 12.0.
+static bool clusters_pay(const Plan& P, uint64_t n) {
+  if (P.cl_clusters == 0 || n == 0) return false;
+  const double steps = (double)n, chunk = std::min(steps, (double)P.cl_chunk);
+  return P.cl_chain_us + std::max(P.cl_ahead_us, 25.0 / steps) + P.cl_chunk_us / chunk +
+             P.cl_call_us / steps < P.half_us;
 }
 
 static shaken_status build_plan(Plan& P, cudaStream_t st) {
@@ -740,7 +760,7 @@ static shaken_status build_plan(Plan& P, cudaStream_t st) {
         const int shape = sliced_shape(H.Gj, ng, (uint64_t)c->n);
         H.sGp = sliced_threads(H.Gj, shape);
         const uint32_t stile = (uint32_t)shk::kSlicedTile / std::min(H.sGp, (uint32_t)shk::kSlicedTile);
-        for (uint32_t half = 0; half < 2 && !in_cluster; ++half) {
+        for (uint32_t half = 0; half < 2; ++half) {
           const uint64_t cut = sliced_cut(c, half, H, shape, stile);
           for (uint64_t w0 = (cut + stile - 1) / stile * stile; w0 > 0; w0 -= stile)
             stiles[fi][half][shape].push_back(
@@ -852,11 +872,12 @@ static shaken_status build_plan(Plan& P, cudaStream_t st) {
     }
     P.fams.push_back(std::move(F));
   }
-  if (!cds.empty()) TRY(upload(P.ctxlist, cds.data(), cds.size() * sizeof(CtxDev*), st));
+  P.n_rest = (int)cds.size();
+  cds.insert(cds.end(), cl_cds.begin(), cl_cds.end());
+  TRY(upload(P.ctxlist, cds.data(), cds.size() * sizeof(CtxDev*), st));
   P.n_ctx = (int)cds.size();
   if (P.cl_clusters > 0) {
     TRY(upload(P.cl_jobs, ojobs[0].data(), ojobs[0].size() * sizeof(GraphJob), st));
-    TRY(upload(P.cl_ctx, cl_cds.data(), cl_cds.size() * sizeof(CtxDev*), st));
     std::vector<uint32_t> off;
     uint32_t first = 0;
     for (const GraphJob& J : ojobs[0]) {
@@ -885,7 +906,8 @@ static shaken_status graph_obs(const Family& F, int which, int full, cudaStream_
   return SHAKEN_OK;
 }
 
-static shaken_status plan_step_launch(Plan& P, cudaStream_t st, uint64_t* nl,
+// graphs: with the graph members (false: they go in clusters).
+static shaken_status plan_step_launch(Plan& P, cudaStream_t st, uint64_t* nl, bool graphs,
                                       bool capturing = false) {
   uint64_t count = 0;
   const bool timed = P.timing > 0 && !capturing && P.steps_issued % (uint64_t)P.timing == 0;
@@ -897,7 +919,7 @@ static shaken_status plan_step_launch(Plan& P, cudaStream_t st, uint64_t* nl,
     // into half 0 unless a per-step series (which also needs M) is recorded
     if (c->hcd.tracking && c->kind == SHAKEN_LATTICE && c->enc == SHAKEN_MULTISPIN)
       lattice_sums = true;
-    if (c->kind == SHAKEN_GRAPH && P.cl_clusters > 0) continue;  // tracked in its own run
+    if (c->kind == SHAKEN_GRAPH && !graphs) continue;  // tracked in its own run
     if (c->hcd.tracking && c->kind == SHAKEN_GRAPH && c->hcd.record) graph_sums = true;
     if (c->hcd.tracking && c->kind == SHAKEN_GRAPH && !c->hcd.record) track = true;
     ex |= c->exact_always;
@@ -913,6 +935,7 @@ static shaken_status plan_step_launch(Plan& P, cudaStream_t st, uint64_t* nl,
   }
   for (uint32_t half = 0; half < 2; ++half) {
     for (auto& F : P.fams) {
+      if (F->kind == 1 && !graphs) continue;
       cudaEvent_t e0 = nullptr, e1 = nullptr;
       if (timed) {
         e0 = P.get_event();
@@ -951,7 +974,7 @@ static shaken_status plan_step_launch(Plan& P, cudaStream_t st, uint64_t* nl,
       }
     }
   }
-  CU(shk::launch_epilogue(P.ctxlist.as<CtxDev*>(), P.n_ctx, st));
+  CU(shk::launch_epilogue(P.ctxlist.as<CtxDev*>(), graphs ? P.n_ctx : P.n_rest, st));
   ++count;
   *nl += count;
   return SHAKEN_OK;
@@ -961,9 +984,10 @@ static constexpr int kGraphChunk = 32;
 
 // Full steps that a run of a plan has issued: members in clusters, and the others.
 struct Issued {
+  bool in_clusters = false;  // the graph members
   uint64_t clusters = 0, rest = 0;
-  uint64_t of(const Plan& P, const shaken_ctx* c) const {
-    return c->kind == SHAKEN_GRAPH && P.cl_clusters > 0 ? clusters : rest;
+  uint64_t of(const shaken_ctx* c) const {
+    return c->kind == SHAKEN_GRAPH && in_clusters ? clusters : rest;
   }
 };
 
@@ -977,7 +1001,8 @@ static shaken_status may_issue(Plan& P) {
 static shaken_status plan_run(Plan& P, cudaStream_t st, uint64_t n_steps, bool use_graph,
                               uint64_t* nl, Issued* issued) {
   if (P.dirty) TRY(build_plan(P, st));
-  if (P.cl_clusters > 0) {
+  bool clusters = clusters_pay(P, n_steps);
+  if (clusters) {
     const size_t work =
         shk::graph_cluster_step_bytes(P.cl_classes, P.cl_clusters, P.cl_passes) *
         (size_t)std::min<uint64_t>(n_steps, P.cl_chunk);
@@ -986,23 +1011,31 @@ static shaken_status plan_run(Plan& P, cudaStream_t st, uint64_t n_steps, bool u
     while (room < work) room *= 2;
     if (P.cl_work.bytes < work && P.cl_work.alloc(room) != SHAKEN_OK) {
       P.cl_refused = true;  // the half-step kernels take no such buffer
-      TRY(build_plan(P, st));
+      P.cl_clusters = 0;
+      clusters = false;
     }
   }
-  if (P.cl_clusters > 0) {
+  issued->in_clusters = clusters;
+  if (clusters) {
     while (issued->clusters < n_steps) {
       const uint64_t chunk = std::min<uint64_t>(n_steps - issued->clusters, P.cl_chunk);
       TRY(may_issue(P));
       CU(shk::launch_graph_cluster(P.cl_jobs.as<GraphJob>(), P.cl_off.as<uint32_t>(), P.cl_clusters,
                                    P.cl_n, P.cl_m, P.cl_classes, P.cl_passes, P.cl_blocks,
-                                   P.cl_ctx.as<CtxDev*>(), P.cl_n_ctx, (uint32_t)chunk,
-                                   P.cl_work.p, st));
+                                   P.ctxlist.as<CtxDev*>() + P.n_rest, P.cl_n_ctx,
+                                   (uint32_t)chunk, P.cl_work.p, st));
       *nl += 4;
       issued->clusters += chunk;
     }
-    if (P.n_ctx == 0) return SHAKEN_OK;  // no other members
+    if (P.n_rest == 0) return SHAKEN_OK;  // no other members
   }
   if (use_graph && n_steps >= (uint64_t)kGraphChunk) {
+    // the captured steps are of one set of families
+    const int what = (clusters ? 1 : 0) | (P.on_bits ? 2 : 0);
+    if (P.gexec && P.graph_what != what) {
+      CU(cudaStreamSynchronize(st));
+      P.drop_graph();
+    }
     if (!P.gexec) {
       cudaStream_t cap = nullptr;
       CU(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
@@ -1015,7 +1048,7 @@ static shaken_status plan_run(Plan& P, cudaStream_t st, uint64_t n_steps, bool u
       uint64_t cnt = 0;
       shaken_status s = SHAKEN_OK;
       for (int k = 0; k < kGraphChunk && s == SHAKEN_OK; ++k)
-        s = plan_step_launch(P, cap, &cnt, true);
+        s = plan_step_launch(P, cap, &cnt, !clusters, true);
       cudaGraph_t g = nullptr;
       e = cudaStreamEndCapture(cap, &g);
       cudaStreamDestroy(cap);
@@ -1034,6 +1067,7 @@ static shaken_status plan_run(Plan& P, cudaStream_t st, uint64_t n_steps, bool u
         return fail(SHAKEN_E_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
       }
       P.graph = g;
+      P.graph_what = what;
       P.graph_steps = kGraphChunk;
       P.graph_launches = cnt;
     }
@@ -1046,7 +1080,7 @@ static shaken_status plan_run(Plan& P, cudaStream_t st, uint64_t n_steps, bool u
   }
   for (; issued->rest < n_steps; ++issued->rest) {
     shaken_status s = may_issue(P);
-    if (s == SHAKEN_OK) s = plan_step_launch(P, st, nl);
+    if (s == SHAKEN_OK) s = plan_step_launch(P, st, nl, !clusters);
     if (s != SHAKEN_OK) {  // the step is not taken: nor are its sums, if its first half added some
       for (shaken_ctx* c : P.members)
         cudaMemsetAsync(c->step_sums.p, 0, c->step_sums.bytes, st);
@@ -1645,7 +1679,9 @@ static shaken_status run_bits(shaken_ctx* c, uint64_t n_steps, uint64_t* nl, Iss
   uint32_t* w = c->bits.as<uint32_t>();
   CU(shk::launch_bits(1, c->A.as<uint4>(), w, nullptr, words, st));
   std::swap(c->solo.fams, c->solo.bits);
+  c->solo.on_bits = true;
   const shaken_status s = plan_run(c->solo, st, n_steps, n_steps >= 64, nl, issued);
+  c->solo.on_bits = false;
   std::swap(c->solo.fams, c->solo.bits);
   *nl += 1;
   if (issued->rest == 0) return s;  // no step taken: the bytes are the state
@@ -1672,7 +1708,7 @@ static shaken_status solo_run(shaken_ctx* ctx, uint64_t n_steps) {
       bits ? run_bits(ctx, n_steps, &nl, &issued)
            : plan_run(ctx->solo, ctx->stream, n_steps, n_steps >= 64, &nl, &issued);
   ctx->launches += nl;
-  ctx->host_step += issued.of(ctx->solo, ctx);
+  ctx->host_step += issued.of(ctx);
   return s;
 }
 
@@ -2232,7 +2268,7 @@ shaken_status shaken_batch_step(shaken_batch* b, uint64_t n_steps, int use_graph
   Issued issued;
   const shaken_status s = plan_run(b->plan, b->stream, n_steps, use_graph != 0, &nl, &issued);
   b->launches += nl;
-  for (shaken_ctx* c : b->plan.members) c->host_step += issued.of(b->plan, c);
+  for (shaken_ctx* c : b->plan.members) c->host_step += issued.of(c);
   return s;
 }
 
