@@ -14,6 +14,12 @@
  *     caller passes is referenced after a call returns.
  *   - Device memory is allocated and owned by the library (cudaMalloc) and is
  *     released by shaken_free / shaken_batch_free / shaken_server_free.
+ *     Beside the state, whole runs keep scratch from their first run until then:
+ *     outcome words of at most 48 MB for a small INT8/PACKED lattice and 64 MB for
+ *     a context or batch of small +-1 graphs (a server counts them in its budget),
+ *     a quarter of sigma's bytes for an INT8 lattice whose half
+ *     steps run on a bit copy, series buffers of at most 8 MB each.  Where it cannot
+ *     be had, the half-step kernels run without it, with the same trajectory.
  *   - A context is used by one host thread at a time; distinct contexts are
  *     independent.  Work is issued on the CUDA stream given at creation
  *     (borrowed, never destroyed; NULL = the legacy default stream).  Calls
@@ -370,7 +376,8 @@ void shaken_batch_free(shaken_batch* b);
 /* the next ones.  Results are the same as running each job alone.            */
 /* ------------------------------------------------------------------------ */
 
-/* Create a server with a device-memory budget (bytes) for job state and a
+/* Create a server with a device-memory budget (bytes) for job state -- and, in
+ * what the running jobs leave of it, the outcome words of whole runs -- and a
  * chunk length (steps per batched launch sequence between admissions). */
 shaken_status shaken_server_create(shaken_server** out, size_t hbm_budget_bytes,
                                    uint32_t chunk_steps, void* cuda_stream);

@@ -188,6 +188,10 @@ struct Family {
   }
 };
 
+// Bytes of a chunk's outcome words, at most: they stay in L2.  (Chunks of 64 steps instead of what
+// fits, up to 256: 500 annealed steps of n = 2000 2.17 -> 2.42 ms, and the first run no shorter.)
+static constexpr size_t kClusterWork = 64u << 20;
+
 struct Plan {
   std::vector<shaken_ctx*> members;
   std::vector<std::unique_ptr<Family>> fams;
@@ -204,6 +208,7 @@ struct Plan {
   uint32_t cl_n = 0, cl_passes = 0, cl_chunk = 0;
   uint64_t cl_m = 0;
   double cl_chain_us = 0.0, cl_ahead_us = 0.0, cl_chunk_us = 0.0, cl_call_us = 0.0, half_us = 0.0;
+  size_t cl_limit = kClusterWork;  // bytes cl_work may take (a server's: what its jobs leave of the budget)
   bool cl_refused = false;  // no memory for cl_work
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
@@ -581,10 +586,6 @@ static shaken_status choose_lattice_shape(const Plan& P, int enc, const std::vec
   return SHAKEN_OK;
 }
 
-// Bytes of a chunk's outcome words, at most: they stay in L2.  (Chunks of 64 steps instead of what
-// fits, up to 256: 500 annealed steps of n = 2000 2.17 -> 2.42 ms, and the first run no shorter.)
-static constexpr size_t kClusterWork = 64u << 20;
-
 // Whether the graph members of a plan can be stepped in whole runs by graph_cluster_kernel -- +-1
 // couplings, one lambda, every vertex and half step within the bit-sliced kernel -- and long runs
 // take less time per step that way than with the half-step kernels and the epilogue.  The run
@@ -626,7 +627,7 @@ static void choose_clusters(Plan& P) {
   if (passes > 1u << 20 || classes > 32) return;
   const int blocks = shk::graph_cluster_shape(most, edges, classes, clusters, &us);
   const size_t step = shk::graph_cluster_step_bytes(classes, clusters, (uint32_t)passes);
-  const uint32_t chunk = (uint32_t)std::min<size_t>(kClusterWork / step, 256);
+  const uint32_t chunk = (uint32_t)std::min<size_t>(P.cl_limit / step, 256);
   if (blocks == 0 || chunk == 0) return;
   P.cl_chain_us = us;
   P.cl_ahead_us = 2.9e-5 * outcomes;
@@ -1006,10 +1007,12 @@ static shaken_status plan_run(Plan& P, cudaStream_t st, uint64_t n_steps, bool u
     const size_t work =
         shk::graph_cluster_step_bytes(P.cl_classes, P.cl_clusters, P.cl_passes) *
         (size_t)std::min<uint64_t>(n_steps, P.cl_chunk);
-    // with room for a batch that grows by members
+    // with room for a batch that grows by members, if there is
     size_t room = 1u << 20;
     while (room < work) room *= 2;
-    if (P.cl_work.bytes < work && P.cl_work.alloc(room) != SHAKEN_OK) {
+    room = std::max(work, std::min(room, P.cl_limit));
+    if (P.cl_work.bytes < work && P.cl_work.alloc(room) != SHAKEN_OK &&
+        P.cl_work.alloc(work) != SHAKEN_OK) {
       P.cl_refused = true;  // the half-step kernels take no such buffer
       P.cl_clusters = 0;
       clusters = false;
@@ -2546,6 +2549,16 @@ static std::deque<int64_t>::iterator server_pick(shaken_server* s) {
   return Q.end();
 }
 
+// The outcome words of graph clusters take what the states (extra: of a job about to be admitted)
+// leave of the budget; a buffer above that is given back before the job's memory is allocated.
+// Between chunks only: the stream is idle.
+static void server_bound_work(shaken_server* s, size_t extra) {
+  Plan& P = s->batch.plan;
+  const size_t states = s->used + extra;
+  P.cl_limit = std::min(kClusterWork, s->budget > states ? s->budget - states : (size_t)0);
+  if (P.cl_work.bytes > P.cl_limit) P.cl_work.release();
+}
+
 static void server_loop(shaken_server* s) {
   std::unique_lock<std::mutex> lk(s->mu);
   while (true) {
@@ -2556,6 +2569,7 @@ static void server_loop(shaken_server* s) {
       for (auto jt = s->queue.begin(); jt != it; ++jt) s->jobs[*jt]->skips++;
       ServerJob* j = s->jobs[*it].get();
       s->queue.erase(it);
+      server_bound_work(s, j->bytes);
       lk.unlock();
       shaken_ctx* c = j->prepared.release();
       c->stream = s->stream;
@@ -2596,6 +2610,7 @@ static void server_loop(shaken_server* s) {
     }
     // step every running job one chunk
     uint64_t chunk = s->chunk;
+    server_bound_work(s, 0);
     lk.unlock();
     uint64_t nl = 0;
     Issued issued;
