@@ -17,9 +17,10 @@
  *     Beside the state, whole runs keep scratch from their first run until then:
  *     outcome words of at most 48 MB for a small INT8/PACKED lattice and 64 MB for
  *     a context or batch of small +-1 graphs (a server counts them in its budget),
- *     a quarter of sigma's bytes for an INT8 lattice whose half
- *     steps run on a bit copy, series buffers of at most 8 MB each.  Where it cannot
- *     be had, the half-step kernels run without it, with the same trajectory.
+ *     a quarter of sigma's bytes for an INT8 lattice whose half steps run on a bit
+ *     copy, series buffers of at most 8 MB each.  Outcome words and bit copies take
+ *     at most a quarter of the free memory; beyond that other kernels run without
+ *     them, with the same trajectory.
  *   - A context is used by one host thread at a time; distinct contexts are
  *     independent.  Work is issued on the CUDA stream given at creation
  *     (borrowed, never destroyed; NULL = the legacy default stream).  Calls

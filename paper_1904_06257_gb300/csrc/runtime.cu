@@ -141,6 +141,17 @@ struct DevMem {
     bytes = n;
     return SHAKEN_OK;
   }
+  // Scratch that a run can do without: at most a quarter of the free memory, so that what a caller
+  // has planned for still fits beside it.
+  shaken_status alloc_scratch(size_t n) {
+    size_t free_bytes = 0, total = 0;
+    release();
+    if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess || n > free_bytes / 4) {
+      cudaGetLastError();
+      return fail(SHAKEN_E_NOMEM, "scratch of " + std::to_string(n) + " bytes: too little memory");
+    }
+    return alloc(n);
+  }
   shaken_status reserve(size_t n) { return p != nullptr && bytes >= n ? SHAKEN_OK : alloc(n); }
   template <class T>
   T* as() const {
@@ -1011,8 +1022,8 @@ static shaken_status plan_run(Plan& P, cudaStream_t st, uint64_t n_steps, bool u
     size_t room = 1u << 20;
     while (room < work) room *= 2;
     room = std::max(work, std::min(room, P.cl_limit));
-    if (P.cl_work.bytes < work && P.cl_work.alloc(room) != SHAKEN_OK &&
-        P.cl_work.alloc(work) != SHAKEN_OK) {
+    if (P.cl_work.bytes < work && P.cl_work.alloc_scratch(room) != SHAKEN_OK &&
+        P.cl_work.alloc_scratch(work) != SHAKEN_OK) {
       P.cl_refused = true;  // the half-step kernels take no such buffer
       P.cl_clusters = 0;
       clusters = false;
@@ -1552,7 +1563,7 @@ static bool cluster_eligible(shaken_ctx* c, uint64_t n_steps) {
 static uint32_t ahead_chunk(shaken_ctx* c, int nc, int n_jobs, uint32_t words, uint64_t n_steps) {
   size_t bytes = 0;
   const uint32_t chunk = shk::lattice_ahead_chunk(nc, n_jobs, words, n_steps, &bytes);
-  if (chunk == 0 || (c->ahead.bytes < bytes && c->ahead.alloc(bytes) != SHAKEN_OK)) return 0;
+  if (chunk == 0 || (c->ahead.bytes < bytes && c->ahead.alloc_scratch(bytes) != SHAKEN_OK)) return 0;
   return chunk;
 }
 
@@ -1704,7 +1715,7 @@ static shaken_status solo_run(shaken_ctx* ctx, uint64_t n_steps) {
   Issued issued;
   bool bits = bits_eligible(ctx, n_steps);
   if (bits && ctx->bits.p == nullptr) {  // no memory for the copy: on the bytes
-    bits = ctx->bits.alloc(ctx->spin_bytes / 4) == SHAKEN_OK;
+    bits = ctx->bits.alloc_scratch(ctx->spin_bytes / 4) == SHAKEN_OK;
     if (bits) ctx->solo.invalidate();
   }
   const shaken_status s =
