@@ -668,6 +668,14 @@ static bool clusters_pay(const Plan& P, uint64_t n) {
              P.cl_call_us / steps < P.half_us;
 }
 
+// Whether the graphs' first half steps add up the energies of sigma_t themselves (a recorded run
+// takes them, with M, from the observables kernel).
+static bool fused_tracking(const Plan& P) {
+  for (const shaken_ctx* c : P.members)
+    if (c->kind == SHAKEN_GRAPH && c->hcd.tracking && !c->hcd.record) return true;
+  return false;
+}
+
 static shaken_status build_plan(Plan& P, cudaStream_t st) {
   // the families of the last build keep their device buffers (a plan is rebuilt at the beginning
   // and the end of every anneal and recorded run: 30 us of allocations each time otherwise)
@@ -861,7 +869,7 @@ static shaken_status build_plan(Plan& P, cudaStream_t st) {
     for (int half = 0; half < 2; ++half) {
       for (int k = 0; k < shk::kSlicedShapes; ++k) {
         std::vector<Tile>& sl = stiles[fi][half][k];
-        if (!sl.empty()) deal_tiles(sl, shk::graph_sliced_blocks(k, half == 0));
+        if (!sl.empty()) deal_tiles(sl, shk::graph_sliced_blocks(k, half == 0 && fused_tracking(P)));
         F->stiles[half][k] = put(sl);
       }
       F->gtiles[half] = put(gtiles[fi][half]);
@@ -924,7 +932,8 @@ static shaken_status plan_step_launch(Plan& P, cudaStream_t st, uint64_t* nl, bo
   uint64_t count = 0;
   const bool timed = P.timing > 0 && !capturing && P.steps_issued % (uint64_t)P.timing == 0;
   if (!capturing) ++P.steps_issued;
-  bool lattice_sums = false, graph_sums = false, track = false;
+  bool lattice_sums = false, graph_sums = false;
+  const bool track = fused_tracking(P);
   int ex = 0;
   for (shaken_ctx* c : P.members) {
     // multispin lattices track with the observables kernel; graphs fuse tracking
@@ -933,7 +942,6 @@ static shaken_status plan_step_launch(Plan& P, cudaStream_t st, uint64_t* nl, bo
       lattice_sums = true;
     if (c->kind == SHAKEN_GRAPH && !graphs) continue;  // tracked in its own run
     if (c->hcd.tracking && c->kind == SHAKEN_GRAPH && c->hcd.record) graph_sums = true;
-    if (c->hcd.tracking && c->kind == SHAKEN_GRAPH && !c->hcd.record) track = true;
     ex |= c->exact_always;
   }
   for (auto& F : P.fams) {
