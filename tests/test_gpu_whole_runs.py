@@ -1,4 +1,7 @@
-"""Whole runs in one launch per chunk: what a call promises besides its trajectory."""
+"""Whole runs in one launch per chunk: what a call promises besides its trajectory (it returns before the GPU is done
+where the header says so, counts every kernel it launches, leaves a countable state when a chunk is refused), and what
+is carried over the end of a chunk: m, H, best energies and their steps, against the same steps taken one at a time
+by the half-step kernels."""
 import numpy as np
 import pytest
 
@@ -155,3 +158,55 @@ def test_refused_chunk_of_a_batch(S, after):
         S.shaken_free(ref)
         S.shaken_free(c)
     S.shaken_batch_free(b)
+
+
+def small_problem(S, kind):
+    if kind == "graph":
+        n = 500
+        u, v = W.erdos_renyi(n, 6.0, 3)
+        return graph_problem(S, n, u, v, W.couplings_pm1(u.size, 4), 32, 0.8), 32, n
+    if kind == "multispin":
+        return lattice_problem(S, S.MULTISPIN, 64, 64, W.beta_grid(64)), 64, 64 * 64
+    return lattice_problem(S, S.INT8 if kind == "int8" else S.PACKED, 64, 2, [0.4, 0.5], q=0.7), 2, 64 * 64
+
+
+@pytest.mark.parametrize("kind", ["graph", "multispin", "int8", "packed"])
+def test_recorded_runs_across_chunks_equal_single_steps(S, kind):
+    n = 300  # chunks of 128 or 256 steps
+    p, R, sites = small_problem(S, kind)
+    c = S.shaken_init(p, 11)
+    S.shaken_step(c, 3)
+    m, H = S.shaken_step_record(c, n, R)
+    end = S.shaken_observables(c, R), S.shaken_get_spins(c, R, sites), S.shaken_get_spins_prime(c, R, sites)
+    S.shaken_free(c)
+    c = S.shaken_init(p, 11)
+    S.shaken_step(c, 3)
+    for k in range(n):
+        m1, H1 = S.shaken_step_record(c, 1, R)
+        assert np.array_equal(m1[0], m[k]) and np.array_equal(H1[0], H[k]), k
+    ref = S.shaken_observables(c, R), S.shaken_get_spins(c, R, sites), S.shaken_get_spins_prime(c, R, sites)
+    S.shaken_free(c)
+    for f in ("energy", "pair_energy", "best_energy", "best_step"):
+        assert np.array_equal(end[0][f], ref[0][f]), f
+    assert np.array_equal(end[1], ref[1]) and np.array_equal(end[2], ref[2])
+    low = np.minimum(H.min(axis=0), ref[0]["energy"])
+    assert np.array_equal(ref[0]["best_energy"], low)
+    first = np.where(H.min(axis=0) <= low, 3 + H.argmin(axis=0), n + 3)
+    assert np.array_equal(ref[0]["best_step"], first)
+
+
+@pytest.mark.parametrize("kind", ["graph", "multispin", "int8", "packed"])
+def test_anneals_across_chunks_equal_single_steps(S, kind):
+    """Best energy and its step of an anneal of 300 steps against 300 anneals of one step each."""
+    p, R, sites = small_problem(S, kind)
+    sched = W.linear_schedule(0.1, 2.5, 300)
+    ends = []
+    for pieces in ([sched], [[b] for b in sched]):
+        c = S.shaken_init(p, 12)
+        for s in pieces:
+            S.shaken_anneal(c, s)
+        obs = S.shaken_observables(c, R)
+        ends.append((obs["best_energy"], obs["best_step"], S.shaken_get_spins(c, R, sites)))
+        S.shaken_free(c)
+    for a, b in zip(*ends):
+        assert np.array_equal(a, b)
