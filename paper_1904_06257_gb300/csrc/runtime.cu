@@ -1624,8 +1624,9 @@ static shaken_status run_cluster(shaken_ctx* c, uint64_t n_steps) {
   shaken_status s = SHAKEN_OK;
   while (s == SHAKEN_OK && done < n_steps) s = next();
   c->host_step += done;
-  if (done == 0) return s;
   // the device step counter follows on the stream: the call returns before the run is done
+  // (anneals and recorded runs, which wait for it, write the counter at their end)
+  if (done == 0 || c->hcd.record || c->hcd.anneal_len != 0) return s;
   CU(shk::launch_advance(c->solo.ctxlist.as<CtxDev*>(), 1, (uint32_t)done, st));
   c->launches++;
   return s;
