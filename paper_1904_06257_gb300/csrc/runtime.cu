@@ -221,6 +221,7 @@ struct Plan {
   double cl_chain_us = 0.0, cl_ahead_us = 0.0, cl_chunk_us = 0.0, cl_call_us = 0.0, half_us = 0.0;
   size_t cl_limit = kClusterWork;  // bytes cl_work may take (a server's: what its jobs leave of the budget)
   bool cl_refused = false;  // no memory for cl_work
+  bool half_tiles = false;  // the half-step tiles of members in clusters, too (once a short call needs them)
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
   int graph_what = 0;  // what the captured steps are of (plan_run)
@@ -780,7 +781,7 @@ static shaken_status build_plan(Plan& P, cudaStream_t st) {
         const int shape = sliced_shape(H.Gj, ng, (uint64_t)c->n);
         H.sGp = sliced_threads(H.Gj, shape);
         const uint32_t stile = (uint32_t)shk::kSlicedTile / std::min(H.sGp, (uint32_t)shk::kSlicedTile);
-        for (uint32_t half = 0; half < 2; ++half) {
+        for (uint32_t half = 0; half < 2 && (!in_cluster || P.half_tiles); ++half) {
           const uint64_t cut = sliced_cut(c, half, H, shape, stile);
           for (uint64_t w0 = (cut + stile - 1) / stile * stile; w0 > 0; w0 -= stile)
             stiles[fi][half][shape].push_back(
@@ -1033,9 +1034,13 @@ static shaken_status plan_run(Plan& P, cudaStream_t st, uint64_t n_steps, bool u
     if (P.cl_work.bytes < work && P.cl_work.alloc_scratch(room) != SHAKEN_OK &&
         P.cl_work.alloc_scratch(work) != SHAKEN_OK) {
       P.cl_refused = true;  // the half-step kernels take no such buffer
-      P.cl_clusters = 0;
+      TRY(build_plan(P, st));
       clusters = false;
     }
+  }
+  if (!clusters && P.cl_clusters > 0 && !P.half_tiles) {
+    P.half_tiles = true;
+    TRY(build_plan(P, st));
   }
   issued->in_clusters = clusters;
   if (clusters) {
