@@ -18,8 +18,8 @@
 // What bounds it: integer issue.  A LOP3, a PRMT and a wide product each hold the SM
 // quarter's common issue port for two cycles (a product and k logic operations take
 // max(4, 2 + 2k) cycles), so a word of the Erdos-Renyi graph (mean degree 8, n = 10^6,
-// 256 replicas) with its ~300 such operations needs 600 cycles: 120 us a half step, of
-// which 178 us are reached (ALU pipe 56 %, issue 51 %, 1720 warp instructions per
+// 256 replicas) with its ~300 such operations needs 600 cycles: a bound of 120 us a half
+// step, measured 178 us (ALU pipe 56 %, issue 51 %, 1720 warp instructions per
 // 4-word thread, next: gathers).  The general kernel's byte counters, byte lookups and
 // bit transposes take 907 instructions a word and 370 us; with tracking 238 against
 // 412 us.  Four words a thread (16 warps an SM at 128 registers) against two (20 warps):

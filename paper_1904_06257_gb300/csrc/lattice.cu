@@ -653,11 +653,11 @@ __global__ void __launch_bounds__(kTile) lattice_resident_kernel(const LatJob* _
         if (stab.collapsed) {
           Lw = classify<true>(S, V, H, F, stab);
           decide_head3<true>(Lw, stab, K, P, w, half, calls);
-          decide_tail<true>(Lw, stab, K, P, w, half, 3u, calls);
+          decide_tail<true>(Lw, stab, K, P, w, half, 3u);
         } else {
           Lw = classify<false>(S, V, H, F, stab);
           decide_head3<false>(Lw, stab, K, P, w, half, calls);
-          decide_tail<false>(Lw, stab, K, P, w, half, 3u, calls);
+          decide_tail<false>(Lw, stab, K, P, w, half, 3u);
         }
         out[w] = Lw.res;
         if (track && pos == 0u) {
@@ -972,7 +972,7 @@ __device__ __forceinline__ void band_edge(const LatJob& J, const LatTable& tab,
     const uint32_t F = J.frozen != nullptr ? J.frozen[a] : 0u;
     LaneWord L = classify<COLL>(S, V, H, F, tab);
     decide_head3<COLL>(L, tab, K, P, a, typ, calls);
-    if (L.U != 0u) decide_tail<COLL>(L, tab, K, P, a, typ, 3u, calls);
+    if (L.U != 0u) decide_tail<COLL>(L, tab, K, P, a, typ, 3u);
     out[wpr + oo] = L.res;
     st_relaxed_u64(pub + c, tag | L.res);
   }

@@ -97,7 +97,6 @@ __global__ void __launch_bounds__(kClusterThreads, 1) lattice_cluster_kernel(
     for (uint32_t k = 0; k < 3u; ++k) W[k] = ph_call_shared(K, P, w_first + tid, typ + 2u * k);
   };
   call_ahead(order);
-  uint32_t calls = 0;
 #pragma unroll 1
   for (uint32_t hs = 0; hs < 2u * n_steps; ++hs) {
     const uint32_t pos = hs & 1u, typ = pos ^ order, nxt = typ ^ 1u, t = t0 + (hs >> 1);
@@ -140,11 +139,11 @@ __global__ void __launch_bounds__(kClusterThreads, 1) lattice_cluster_kernel(
       if (tab.collapsed) {
         Lw = classify<true>(S, V, H, F, tab);
         decide_planes3<true>(Lw, tab, W);
-        decide_tail<true>(Lw, tab, K, P, w, typ, 3u, calls);
+        decide_tail<true>(Lw, tab, K, P, w, typ, 3u);
       } else {
         Lw = classify<false>(S, V, H, F, tab);
         decide_planes3<false>(Lw, tab, W);
-        decide_tail<false>(Lw, tab, K, P, w, typ, 3u, calls);
+        decide_tail<false>(Lw, tab, K, P, w, typ, 3u);
       }
       const uint32_t res = Lw.res;
       out[o] = res;
@@ -188,7 +187,6 @@ __global__ void __launch_bounds__(kClusterThreads, 1) lattice_cluster_kernel(
     static_cast<uint32_t*>(J.A)[w_first + o] = smem[o];
     static_cast<uint32_t*>(J.B)[w_first + o] = smem[own + o];
   }
-  (void)calls;
   if (!track || r != 0u) return;
   // block 0: m and H of every step of the chunk, lane k replica k; the first of the least H
   const double Jc = cd->Jc, lam2 = 2.0 * cd->lamc, inv_n = cd->inv_n;

@@ -241,11 +241,10 @@ __device__ __forceinline__ void decide_head_words(LaneWord (&Lw)[WPT], const Lat
 template <bool COLL>
 __device__ __forceinline__ void decide_tail(LaneWord& L, const LatTable& tab, const PhKey& K,
                                             const PhShared& P, uint32_t a, uint32_t half,
-                                            uint32_t first, uint32_t& calls) {
+                                            uint32_t first) {
 #pragma unroll 1
   for (uint32_t call = first; call < 8 && L.U != 0u; ++call) {
     const uint4 w = ph_call_shared(K, P, a, half + 2u * call);
-    ++calls;
     apply_call<COLL>(L, w, tab, call);
   }
 }
