@@ -496,7 +496,7 @@ def run_ours(args, rank, world, local_rank):
 # ------------------------------------------------------------------------ traffic
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic.json")
 KERNEL_SOURCES = [os.path.join(ROOT, "paper_1904_06257_gb300", "csrc", f)
-                  for f in ("lattice.cu", "shaken_internal.cuh")]
+                  for f in ("lattice.cu", "lattice_device.cuh", "shaken_internal.cuh")]
 
 
 MICROBENCH_KINDS = ("philox_calls", "lop3", "imad", "lop3_imad_mix", "mad_wide", "mul_wide",
